@@ -431,7 +431,9 @@ typedef struct {
   double tol;           /* target FP64 ||b - D x|| / ||b|| (e.g. 1e-10) */
   int max_iter;         /* cap on iterations (CGNE) / inner FGCR iterations (MG) */
   int gcr_m;            /* FGCR restart length (MG) */
-  int nu;               /* MR smoothing steps after the coarse correction (MG) */
+  int nu;               /* MR smoothing steps on D after the coarse correction (MG); with
+                           every extent even, (nu + 1) / 2 steps on the even-odd
+                           operator stand for them */
   double inner_tol;     /* relative reduction asked of each FP32 cycle (MG) */
   double coarse_tol;    /* relative tolerance of the preconditioner's coarse solve */
   int coarse_max_iter;  /* cap on coarse iterations per preconditioner call */

@@ -388,6 +388,9 @@ void mglma_gauge_free(mglma_gauge G) {
   cudaFree(G->Cinv64);
   cudaFree(G->Udf);
   cudaFree(G->Cdf);
+  cudaFree(G->Ueo);
+  cudaFree(G->Ceo);
+  cudaFree(G->Ieo);
   delete G;
 }
 

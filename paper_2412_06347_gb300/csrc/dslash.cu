@@ -1139,10 +1139,13 @@ mglma_status dslash_gcr(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& in,
         <<<(unsigned)(nblk * in.nrhs), 128, 0, s>>>(in.p, out.p, G->U32, G->C32, a, nullptr, MrArgs(), gd);
   }
   MG_LAUNCH_CHECK();
-  {
-    ProfScope ps(ctx, K_REDUCE, s, (double)dslash_gcr_part_doubles(in.V, in.nrhs) * 8.0);
-    gd_finish_kernel<<<in.nrhs, 256, 0, s>>>(part, nblk, k, in.nrhs, nw, num, dots);
-  }
+  return gd_finish(ctx, part, nblk, k, in.nrhs, nw, num, dots, s);
+}
+
+mglma_status gd_finish(mglma_ctx ctx, const double* part, int64_t nblk, int k, int nrhs, double* nw, double2* num,
+                       double2* dots, cudaStream_t s) {
+  ProfScope ps(ctx, K_REDUCE, s, 48.0 * nblk * nrhs);
+  gd_finish_kernel<<<nrhs, 256, 0, s>>>(part, nblk, k, nrhs, nw, num, dots);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }

@@ -92,6 +92,7 @@ struct KernelStat {
 }  // namespace mglma
 
 #include <map>
+#include <mutex>
 #include <tuple>
 
 struct mglma_ctx_s {
@@ -138,6 +139,13 @@ struct mglma_gauge_s {
   double2* Cinv64 = nullptr;  // [2][18][V] inverse clover blocks (even-odd, formed on first use)
   float4* Udf = nullptr;      // [4][9][V] U64 split into double-float (re.hi, re.lo, im.hi, im.lo), first use
   float4* Cdf = nullptr;      // [2][18][V] C64 split likewise (two reals per float4), first use
+  // parity-split FP32 copies of the even-odd stencil (layouts in schur.cu),
+  // formed on first use: links (18 reals, time-boundary sign applied), A_ee and
+  // -1/2 A_oo^-1; eo_state 1 formed, -1 unusable (odd extent, singular block), 0
+  // not tried
+  char *Ueo = nullptr, *Ceo = nullptr, *Ieo = nullptr;
+  int eo_state = 0;
+  std::mutex eo_mu;
   int slabs_loaded = 0;   // time slices received
   std::vector<char> slab_seen;
   bool ready = false;
@@ -286,6 +294,9 @@ size_t dslash_gcr_part_doubles(int64_t V, int nrhs);
 mglma_status dslash_gcr(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, Spinor& out, int k, const void* W0,
                         size_t wslot_reals, const void* res, double* part, double* nw, double2* num, double2* dots,
                         cudaStream_t s);
+// the partials of dslash_gcr / schur_gcr ([rhs][nblk][6]) summed in a fixed order
+mglma_status gd_finish(mglma_ctx, const double* part, int64_t nblk, int k, int nrhs, double* nw, double2* num,
+                       double2* dots, cudaStream_t s);
 // z += alpha s (per-RHS alpha) for BF16 s and FP32 z: the last MR step
 mglma_status mr_zupdate(mglma_ctx, const double2* alpha, const Spinor& sk, Spinor& z, cudaStream_t s);
 mglma_status dslash_mr_step(mglma_ctx, const mglma_gauge_s* G, const Spinor& t, Spinor& tn, Spinor& sk, Spinor& z,
@@ -306,6 +317,53 @@ mglma_status dslash_resid(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, c
 mglma_status dslash_dot(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, Spinor& out, double* part, double* nrm,
                         double2* dot, cudaStream_t s);
 size_t dslash_dot_part_doubles(int64_t V, int nrhs);
+// ---- even-odd FP32 stencil (schur.cu).  Half fields: Spinors of V / 2 sites.
+// Forms the parity-split copies on first use; *usable false (and MGLMA_OK)
+// when an extent is odd, a clover block has no good inverse or memory is short.
+mglma_status fine_eo_ready(mglma_ctx, mglma_gauge_s* G, bool* usable, cudaStream_t s);
+// odd pass: w = A_oo^-1 H_oe in (in FP32 or BF16, w FP32)
+mglma_status schur_odd(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, Spinor& w, cudaStream_t s);
+// x_o = A_oo^-1 (b_o - H_oe x_e); without xe: A_oo^-1 b_o (FP32)
+mglma_status schur_odd_solution(mglma_ctx, const mglma_gauge_s* G, const Spinor* xe, const Spinor& bo, Spinor& xo,
+                                cudaStream_t s);
+// even passes, w = schur_odd(x): S x = A_ee x - H_eo w.  The outputs must not
+// alias the inputs.
+//   schur_prepare: out = be - H_eo vo (FP32)
+//   schur_apply: out = S x (FP32)
+//   schur_resid: out (BF16) = b - S x (FP32 b, x)
+//   schur_dot: out = S x (BF16), alpha[r] = <out, x> / |out|^2
+//   schur_mr_step: tn = t - a S t, sn = sk - a t (a = alpha[r]; BF16), then
+//     alpha_n[r] = <tn, sn> / |tn|^2
+//   mr_iterate: z += sum_{k<ns} alpha_k s_k, ns = 1..4 (s_k BF16 fields
+//     sstride_bytes apart from s0, alpha_k at alpha + k nrhs)
+//   schur_gcr: dslash_gcr for S
+// part: schur_part_doubles(V, nrhs) doubles (V of the full lattice)
+size_t schur_part_doubles(int64_t V, int nrhs);
+mglma_status schur_prepare(mglma_ctx, const mglma_gauge_s* G, const Spinor& be, const Spinor& vo, Spinor& out,
+                           cudaStream_t s);
+mglma_status schur_apply(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out,
+                         cudaStream_t s);
+mglma_status schur_resid(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, const Spinor& b,
+                         Spinor& out, cudaStream_t s);
+mglma_status schur_dot(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out, double* part,
+                       float2* alpha, cudaStream_t s);
+mglma_status schur_mr_step(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& t, Spinor& tn,
+                           const Spinor& sk, Spinor& sn, const float2* alpha, float2* alpha_n, double* part,
+                           cudaStream_t s);
+mglma_status mr_iterate(mglma_ctx, Spinor& z, const void* s0, size_t sstride_bytes, int ns, const float2* alpha,
+                        cudaStream_t s);
+mglma_status schur_gcr(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out, int k,
+                       const void* W0, size_t wslot_reals, const void* r, double* part, double* nw, double2* num,
+                       double2* dots, cudaStream_t s);
+// FP64 full field times scale[rhs] -> FP32 halves; FP32 halves -> FP32 full
+// field f with x (FP64 full) += scale[rhs] f; FP32 even half <-> full field
+// (embed: zero on the odd sites)
+mglma_status eo_split(mglma_ctx, const mglma_gauge_s* G, const Spinor& f, Spinor& e, Spinor& o, const double* scale,
+                      cudaStream_t s);
+mglma_status eo_join(mglma_ctx, const mglma_gauge_s* G, const Spinor& e, const Spinor& o, Spinor& f, Spinor& x,
+                     const double* scale, cudaStream_t s);
+mglma_status eo_embed(mglma_ctx, const mglma_gauge_s* G, const Spinor& e, Spinor& f, cudaStream_t s);
+mglma_status eo_extract(mglma_ctx, const mglma_gauge_s* G, const Spinor& f, Spinor& e, cudaStream_t s);
 // single hop-slot pieces of D in FP64, used to assemble the coarse operator:
 // slot d < 8: the hop term of slot d at sites whose hop leaves their block
 // (zero elsewhere); slot 8: clover term plus every hop that stays in the block.

@@ -251,7 +251,7 @@ static mglma_status read_active(GcrWork& w, int n, std::vector<int>& h) {
 // Batched flexible GCR(m): x = A^-1 b per RHS to |r| <= tol |b| (or max_iter).
 // M (nullable) is the right preconditioner.  poll_every > 0 reads the active
 // mask on the host every that many iterations and stops when all converged.
-// tol_scale (nullable, host, n entries): RHS r stops at |r| <= tol *
+// tol_scale (nullable, host, n entries; unit_ref: see below): RHS r stops at |r| <= tol *
 // tol_scale[r] * |b_r| instead of tol * |b_r|.
 // Graphs of whole FGCR iterations, one per direction slot k, captured on
 // first use; valid while the workspace, the iterate and the operators keep
@@ -268,7 +268,7 @@ struct IterGraphs {
 
 static mglma_status gcr_run(GcrWork& w, const OpFn& A, const OpFn* M, const Vec& b, Vec& x, int max_iter, double tol,
                             int poll_every, GcrResult& res, const std::vector<double>* tol_scale,
-                            IterGraphs* graphs);
+                            IterGraphs* graphs, bool unit_ref = false);
 
 static mglma_status gcr(mglma_ctx ctx, cudaStream_t s, const OpFn& A, const OpFn* M, const Vec& b, Vec& x, int m,
                         int max_iter, double tol, int poll_every, GcrResult& res,
@@ -312,7 +312,7 @@ static mglma_status gcr_iter_graphed(GcrWork& w, const OpFn& A, const OpFn* M, V
 
 static mglma_status gcr_run(GcrWork& w, const OpFn& A, const OpFn* M, const Vec& b, Vec& x, int max_iter, double tol,
                             int poll_every, GcrResult& res, const std::vector<double>* tol_scale,
-                            IterGraphs* graphs) {
+                            IterGraphs* graphs, bool unit_ref) {
   const int n = b.nrhs;
   const int m = w.m;
   cudaStream_t s = w.s;
@@ -325,7 +325,9 @@ static mglma_status gcr_run(GcrWork& w, const OpFn& A, const OpFn* M, const Vec&
     double* bb = w.sc.d + (size_t)(w.m + 1) * w.cap;
     std::vector<double> hb;
     MG_CHECK(read_doubles(bb, hb, n, s));
-    for (int i = 0; i < n; ++i) hb[i] *= (*tol_scale)[i] * (*tol_scale)[i];
+    // unit_ref: the reference is a residual of norm one of which b is a part
+    for (int i = 0; i < n; ++i)
+      hb[i] = (unit_ref ? (hb[i] > 0 ? 1.0 : 0.0) : hb[i]) * (*tol_scale)[i] * (*tol_scale)[i];
     MG_CUDA(cudaMemcpyAsync(bb, hb.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s));
     MG_CUDA(cudaStreamSynchronize(s));
   }
@@ -807,6 +809,10 @@ static Spinor as_spinor(const Vec& v, int64_t V) {
   return f;
 }
 
+// MR steps on the even-odd operator S that stand for nu steps on D (a step on S
+// damps about what two steps on D do)
+static int schur_steps(int nu) { return (nu + 1) / 2; }
+
 // The preconditioner K r = z (FP32): coarse correction then MR smoothing.
 // Scratch is allocated on the first call and reused.
 struct TwoLevel {
@@ -826,7 +832,14 @@ struct TwoLevel {
   bool tc_r0 = false;      // R0 on the tensor cores (BF16 operands; the coarse solve is BF16 already)
   bool tc_t0 = false;      // T0 on the tensor cores (BF16 operands)
   bool capturing = false;  // recording into a graph: the coarse loop runs on the device
+  // even-odd form: r and z are FP32 half fields (even sites) of the Schur
+  // system, the odd part of the full residual being zero
+  bool eo = false;
+  static constexpr int kGroup = 4;  // smoothing steps whose s_k are held at once
+  Vec full, wo;  // a full field for R0 / T0, and A_oo^-1 H_oe of the smoother's vectors
   ~TwoLevel() {
+    dfree(ctx, full.p, s);
+    dfree(ctx, wo.p, s);
     dfree(ctx, b1.p, s);
     dfree(ctx, e1.p, s);
     dfree(ctx, sv.p, s);
@@ -845,7 +858,7 @@ struct TwoLevel {
     // the smoother's s and t: BF16 on the fused path (the flexible outer
     // solve takes the rounded preconditioner; measured: same FGCR and coarse
     // iteration counts as FP32 at 64x32^3), FP32 otherwise
-    fused = p->nu > 1 && dslash_mr_fused(ctx, G, n);
+    fused = eo || (p->nu > 1 && dslash_mr_fused(ctx, G, n));
     tc_r0 = n >= 8 && restrict_tc_supported(C->sub);
     tc_t0 = n >= 8 && prolong_tc_supported(C->sub);
     sv = r;
@@ -853,11 +866,21 @@ struct TwoLevel {
     sv.p = nullptr;
     if (fused) sv.prec = MGLMA_BF16;
     tv = tv2 = sv;
-    MG_CHECK(dalloc(ctx, &sv.p, sv.bytes(), s));
+    MG_CHECK(dalloc(ctx, &sv.p, sv.bytes() * (eo ? std::min(kGroup, std::max(1, schur_steps(p->nu))) : 1), s));
     MG_CHECK(dalloc(ctx, &tv.p, tv.bytes(), s));
     if (fused) MG_CHECK(dalloc(ctx, &tv2.p, tv2.bytes(), s));
-    MG_CHECK(dalloc(ctx, (void**)&part, dslash_dot_part_doubles(C->sub->geo.V, n) * sizeof(double), s));
-    MG_CHECK(sc.alloc(ctx, n, 1, 1, s));
+    if (eo) {
+      wo = full = r;
+      wo.nrhs = full.nrhs = n;
+      wo.p = full.p = nullptr;
+      full.n = 2 * r.n;
+      MG_CHECK(dalloc(ctx, &wo.p, wo.bytes(), s));
+      MG_CHECK(dalloc(ctx, &full.p, full.bytes(), s));
+    }
+    const int64_t V = C->sub->geo.V;
+    MG_CHECK(dalloc(ctx, (void**)&part,
+                    (eo ? schur_part_doubles(V, n) : dslash_dot_part_doubles(V, n)) * sizeof(double), s));
+    MG_CHECK(sc.alloc(ctx, n, 1, eo ? kGroup + 1 : 1, s));
     cs.ctx = ctx;
     cs.s = s;
     cs.C = C;
@@ -877,6 +900,15 @@ struct TwoLevel {
     Vec b1n = b1, e1n = e1, svn = sv, tvn = tv, tv2n = tv2;
     b1n.nrhs = e1n.nrhs = svn.nrhs = tvn.nrhs = tv2n.nrhs = n;
     Spinor rs = as_spinor(r, V), zs = as_spinor(z, V);
+    Spinor rh, zh;  // the half fields
+    if (eo) {
+      rh = as_spinor(r, V / 2);
+      zh = as_spinor(z, V / 2);
+      Vec f = full;
+      f.nrhs = n;
+      rs = zs = as_spinor(f, V);
+      MG_CHECK(eo_embed(ctx, G, rh, rs, s));
+    }
     if (tc_r0)
       MG_CHECK(restrict_tc(ctx, const_cast<mglma_subspace_s*>(S), rs, b1n.p, s));
     else
@@ -889,6 +921,10 @@ struct TwoLevel {
       MG_CHECK(prolong_tc(ctx, const_cast<mglma_subspace_s*>(S), e1n.p, zs, s));
     else
       MG_CHECK(prolong_coarse(ctx, S, e1n.p, zs, false, s));
+    if (eo) {
+      MG_CHECK(eo_extract(ctx, G, zs, zh, s));
+      return smooth_eo(rh, zh, n);
+    }
     if (p->nu > 0) {
       // s = r - D z (in the stencil's epilogue) ; nu MR steps on D e = s,
       // accumulated into z (the last one leaves s as it is)
@@ -921,6 +957,65 @@ struct TwoLevel {
     }
     return MGLMA_OK;
   }
+  Spinor odd_work(int n) const {
+    Vec v = wo;
+    v.nrhs = n;
+    return as_spinor(v, C->sub->geo.V / 2);
+  }
+  // out = S in, and the FGCR image with its dots (see AdFn), on half fields;
+  // the work field exists once the preconditioner ran
+  mglma_status schur(const Spinor& in, Spinor& out) {
+    Spinor w = odd_work(in.nrhs);
+    MG_CHECK(schur_odd(ctx, G, in, w, s));
+    return schur_apply(ctx, G, w, in, out, s);
+  }
+  mglma_status schur_image(const Spinor& in, Spinor& out, int k, const Vec& W0, size_t wslot, const Vec& res,
+                           double* gpart, double* nw, double2* num, double2* dots) {
+    Spinor w = odd_work(in.nrhs);
+    MG_CHECK(schur_odd(ctx, G, in, w, s));
+    return schur_gcr(ctx, G, w, in, out, k, W0.p, wslot, res.p, gpart, nw, num, dots, s);
+  }
+  // s = r - S z, then MR steps on S e = s accumulated into z
+  mglma_status smooth_eo(const Spinor& r, Spinor& z, int n) {
+    const int steps = schur_steps(p->nu);
+    if (steps == 0) return MGLMA_OK;
+    auto half = [&](Vec v) {
+      v.nrhs = n;
+      return as_spinor(v, r.V);
+    };
+    Spinor w = half(wo), ta = half(tv), tb = half(tv2);
+    Spinor *tc = &ta, *tn = &tb;
+    // s_k of up to kGroup steps side by side, alpha_k likewise; z is updated
+    // once per group
+    const size_t stride = sv.bytes();
+    auto slot = [&](int k) {
+      Spinor q = half(sv);
+      q.p = (char*)sv.p + (size_t)(k % kGroup) * stride;
+      return q;
+    };
+    float2* al = reinterpret_cast<float2*>(sc.z);
+    auto alpha = [&](int k) { return al + (size_t)(k % kGroup) * n; };
+    Spinor s0 = slot(0);
+    MG_CHECK(schur_odd(ctx, G, z, w, s));
+    MG_CHECK(schur_resid(ctx, G, w, z, r, s0, s));
+    MG_CHECK(schur_odd(ctx, G, s0, w, s));
+    MG_CHECK(schur_dot(ctx, G, w, s0, *tc, part, alpha(0), s));
+    for (int k = 1; k < steps; ++k) {
+      Spinor sk = slot(k - 1), sn = slot(k);
+      MG_CHECK(schur_odd(ctx, G, *tc, w, s));
+      if (k % kGroup == 0) {
+        // the next slot reuses the group's first: its sum goes into z first,
+        // its last alpha moves out of the way of the new group
+        MG_CHECK(mr_iterate(ctx, z, sv.p, stride, kGroup, al, s));
+        MG_CUDA(cudaMemcpyAsync(al + (size_t)kGroup * n, alpha(k - 1), sizeof(float2) * n, cudaMemcpyDeviceToDevice, s));
+        MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, al + (size_t)kGroup * n, alpha(k), part, s));
+      } else {
+        MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, alpha(k - 1), alpha(k), part, s));
+      }
+      std::swap(tc, tn);
+    }
+    return mr_iterate(ctx, z, sv.p, stride, (steps - 1) % kGroup + 1, al, s);
+  }
 };
 
 // Inner-tolerance factor for a RHS at FP64 relative residual `rel`: when
@@ -940,13 +1035,29 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
   const int64_t V = b.V;
   out.assign(n, RhsStat());
   FreeList fl(ctx, s);
-  Spinor r, r32, e32;
+  // With every extent even the FP32 solve runs on the Schur system of the
+  // even sites (schur.cu): r32 / e32 are then its source and solution (half
+  // fields), ro the odd part of r / |r|, eo the odd part of the correction
+  bool even_odd = false;
+  MG_CHECK(fine_eo_ready(ctx, const_cast<mglma_gauge_s*>(G), &even_odd, s));
+  const int64_t Vs = even_odd ? V / 2 : V;  // sites of the FP32 system
+  Spinor r, r32, e32, re, ro, eo, ef;
   MG_CHECK(alloc_spinor(ctx, r, MGLMA_FP64, n, V, s));
   fl.add(r.p);
-  MG_CHECK(alloc_spinor(ctx, r32, MGLMA_FP32, n, V, s));
+  MG_CHECK(alloc_spinor(ctx, r32, MGLMA_FP32, n, Vs, s));
   fl.add(r32.p);
-  MG_CHECK(alloc_spinor(ctx, e32, MGLMA_FP32, n, V, s));
+  MG_CHECK(alloc_spinor(ctx, e32, MGLMA_FP32, n, Vs, s));
   fl.add(e32.p);
+  if (even_odd) {
+    for (Spinor* f : {&re, &ro, &eo}) {
+      MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP32, n, Vs, s));
+      fl.add(f->p);
+    }
+    MG_CHECK(alloc_spinor(ctx, ef, MGLMA_FP32, n, V, s));
+    fl.add(ef.p);
+  } else {
+    ef = e32;
+  }
   Scalars sc;
   MG_CHECK(sc.alloc(ctx, n, 4, 1, s));
   double* bb = sc.d;
@@ -965,8 +1076,10 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
   K.G = G;
   K.C = C;
   K.p = &p;
+  K.eo = even_odd;
   OpFn A = [&](const Vec& in, Vec& o) {
-    Spinor a = as_spinor(in, V), bo = as_spinor(o, V);
+    Spinor a = as_spinor(in, Vs), bo = as_spinor(o, Vs);
+    if (even_odd) return K.schur(a, bo);
     return dslash(ctx, G, a, bo, false, false, s);
   };
   OpFn Kf = [&](const Vec& in, Vec& o) { return K(in, o); };
@@ -981,11 +1094,13 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
     MG_CHECK(gw.setup(ctx, s, like, n, p.gcr_m));
   }
   double* gpart = nullptr;
-  MG_CHECK(dalloc(ctx, (void**)&gpart, dslash_gcr_part_doubles(V, n) * sizeof(double), s));
+  MG_CHECK(dalloc(ctx, (void**)&gpart,
+                  (even_odd ? schur_part_doubles(V, n) : dslash_gcr_part_doubles(V, n)) * sizeof(double), s));
   fl.add(gpart);
   const AdFn Ad = [&](const Vec& in, Vec& o, int k, const Vec& W0, size_t wslot, const Vec& res, double* nw,
                       double2* num, double2* dots) {
-    Spinor a = as_spinor(in, V), bo = as_spinor(o, V);
+    Spinor a = as_spinor(in, Vs), bo = as_spinor(o, Vs);
+    if (even_odd) return K.schur_image(a, bo, k, W0, wslot, res, gpart, nw, num, dots);
     return dslash_gcr(ctx, G, a, bo, k, W0.p, wslot, res.p, gpart, nw, num, dots, s);
   };
   gw.Ad = &Ad;
@@ -1014,7 +1129,14 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
     MG_CUDA(cudaMemcpyAsync(rr, hrr.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s));
     sqrt_kernel<<<nb, tb, 0, s>>>(rr, rinv, n, 1);
     sqrt_kernel<<<nb, tb, 0, s>>>(rr, rn, n, 0);
-    MG_CHECK(convert_spinor(ctx, r, r32, s, rinv, false));
+    if (even_odd) {
+      // r / |r| on each parity, then b' = r_e - H_eo A_oo^-1 r_o
+      MG_CHECK(eo_split(ctx, G, r, re, ro, rinv, s));
+      MG_CHECK(schur_odd_solution(ctx, G, nullptr, ro, eo, s));
+      MG_CHECK(schur_prepare(ctx, G, re, eo, r32, s));
+    } else {
+      MG_CHECK(convert_spinor(ctx, r, r32, s, rinv, false));
+    }
     Vec v32 = as_vec(r32), e = as_vec(e32);
     // a cycle that can finish a RHS aims at 0.3 tol: a little below what it
     // needs, and no further
@@ -1022,7 +1144,7 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
     for (int i = 0; i < n; ++i) scale[i] = final_cycle_scale(p, out[i].residual);
     GcrResult gr;
     MG_CHECK(gcr_run(gw, A, &Kf, v32, e, p.max_iter - total_inner, p.inner_tol, 1, gr, &scale,
-                     use_graphs ? &graphs : nullptr));
+                     use_graphs ? &graphs : nullptr, even_odd));
     total_inner += gr.iterations;
     for (int i = 0; i < n; ++i) {
       out[i].iterations += gr.per_rhs[i];
@@ -1031,8 +1153,13 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
     // x += |r| e ; r -= |r| D e with D e taken in double-float on the exact
     // FP32 values of e, so r tracks b - D x to about 1e-14 |b| (the FP64
     // products |r| e that enter x are rounded once, below that)
-    MG_CHECK(convert_spinor(ctx, e32, x, s, rn, true));
-    MG_CHECK(dslash_resid_df(ctx, G, e32, r, rn, s));
+    if (even_odd) {
+      MG_CHECK(schur_odd_solution(ctx, G, &e32, ro, eo, s));
+      MG_CHECK(eo_join(ctx, G, e32, eo, ef, x, rn, s));
+    } else {
+      MG_CHECK(convert_spinor(ctx, e32, x, s, rn, true));
+    }
+    MG_CHECK(dslash_resid_df(ctx, G, ef, r, rn, s));
   }
   MG_CHECK(K.cs.take_captured_iters(&K.coarse_iters));
   for (int i = 0; i < n; ++i) out[i].coarse_iterations = K.coarse_iters;
@@ -1139,7 +1266,12 @@ struct Engine {
   MgParams p;
   int cap = 0;
   int64_t V = 0;
-  Spinor b64, x64, r64, r32, e32;
+  // as in mg_solve: with every extent even the FP32 system is the Schur system
+  // of the even sites; ro holds each slot's odd part of r / |r|, te / to / tf
+  // one slot's even, odd and full temporaries
+  bool even_odd = false;
+  int64_t Vs = 0;
+  Spinor b64, x64, r64, r32, e32, ro, te, to, tf;
   double* dsc = nullptr;  // per slot: |r|^2 [cap], |r| [cap], 1/|r| [cap]
   double* stage = nullptr;  // one canonical spinor: host requests pass through it
   double* gpart = nullptr;  // partials of the FGCR image's dots
@@ -1179,14 +1311,25 @@ struct Engine {
       MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP64, cap, V, s));
       fl->add(f->p);
     }
+    MG_CHECK(fine_eo_ready(ctx, const_cast<mglma_gauge_s*>(G), &even_odd, s));
+    Vs = even_odd ? V / 2 : V;
     for (Spinor* f : {&r32, &e32}) {
-      MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP32, cap, V, s));
+      MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP32, cap, Vs, s));
       fl->add(f->p);
+    }
+    if (even_odd) {
+      MG_CHECK(alloc_spinor(ctx, ro, MGLMA_FP32, cap, Vs, s));
+      fl->add(ro.p);
+      for (Spinor* f : {&te, &to, &tf}) {
+        MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP32, 1, f == &tf ? V : Vs, s));
+        fl->add(f->p);
+      }
     }
     MG_CHECK(dalloc(ctx, (void**)&dsc, sizeof(double) * 3 * cap, s));
     fl->add(dsc);
     MG_CHECK(gw.setup(ctx, s, as_vec(r32), cap, p.gcr_m));
-    MG_CHECK(dalloc(ctx, (void**)&gpart, dslash_gcr_part_doubles(V, cap) * sizeof(double), s));
+    MG_CHECK(dalloc(ctx, (void**)&gpart,
+                    (even_odd ? schur_part_doubles(V, cap) : dslash_gcr_part_doubles(V, cap)) * sizeof(double), s));
     fl->add(gpart);
     K.ctx = ctx;
     K.s = s;
@@ -1194,6 +1337,7 @@ struct Engine {
     K.C = C;
     K.p = &p;
     K.cap = cap;
+    K.eo = even_odd;
     MG_CHECK(fill_int(gw.sc.active, 0, cap, s));
     slots.assign(cap, Slot());
     return MGLMA_OK;
@@ -1221,13 +1365,20 @@ struct Engine {
     MG_CUDA(cudaMemcpyAsync(dsc + cap + i, &pr[0], sizeof(double), cudaMemcpyHostToDevice, s));
     MG_CUDA(cudaMemcpyAsync(dsc + 2 * cap + i, &pr[1], sizeof(double), cudaMemcpyHostToDevice, s));
     Spinor rs = ssub(r32, i, 1);
-    MG_CHECK(convert_spinor(ctx, ssub(r64, i, 1), rs, s, dsc + 2 * cap + i, false));
+    if (even_odd) {
+      Spinor roi = ssub(ro, i, 1);
+      MG_CHECK(eo_split(ctx, G, ssub(r64, i, 1), te, roi, dsc + 2 * cap + i, s));
+      MG_CHECK(schur_odd_solution(ctx, G, nullptr, roi, to, s));
+      MG_CHECK(schur_prepare(ctx, G, te, to, rs, s));
+    } else {
+      MG_CHECK(convert_spinor(ctx, ssub(r64, i, 1), rs, s, dsc + 2 * cap + i, false));
+    }
     Vec ri = vsub(as_vec(r32), i, 1), xi = vsub(as_vec(e32), i, 1);
     Vec gr = vsub(gw.view(gw.rp, 0, cap), i, 1);
     double* bb = gw.sc.d + (size_t)(gw.m + 1) * gw.cap;
     MG_CHECK(zero_vec(ctx, xi, s));
     MG_CHECK(copy_vec(ctx, ri, gr, s));
-    // |r32| = 1: the stopping reference is the squared inner-tolerance factor
+    // |r / |r|| = 1: the stopping reference is the squared inner-tolerance factor
     const double sc = final_cycle_scale(p, slots[i].bb > 0 ? rn / std::sqrt(slots[i].bb) : 1.0);
     const double ref = sc * sc;
     MG_CUDA(cudaMemcpyAsync(bb + i, &ref, sizeof(double), cudaMemcpyHostToDevice, s));
@@ -1274,13 +1425,15 @@ struct Engine {
     const int hi = used_prefix();
     if (hi == 0) return MGLMA_OK;
     OpFn A = [&](const Vec& in, Vec& o) {
-      Spinor a = as_spinor(in, V), bo = as_spinor(o, V);
+      Spinor a = as_spinor(in, Vs), bo = as_spinor(o, Vs);
+      if (even_odd) return K.schur(a, bo);
       return dslash(ctx, G, a, bo, false, false, s);
     };
     OpFn M = [&](const Vec& in, Vec& o) { return K(in, o); };
     const AdFn Ad = [&](const Vec& in, Vec& o, int k, const Vec& W0, size_t wslot, const Vec& res, double* nw,
                         double2* num, double2* dots) {
-      Spinor a = as_spinor(in, V), bo = as_spinor(o, V);
+      Spinor a = as_spinor(in, Vs), bo = as_spinor(o, Vs);
+      if (even_odd) return K.schur_image(a, bo, k, W0, wslot, res, gpart, nw, num, dots);
       return dslash_gcr(ctx, G, a, bo, k, W0.p, wslot, res.p, gpart, nw, num, dots, s);
     };
     gw.Ad = &Ad;
@@ -1298,7 +1451,13 @@ struct Engine {
       if (act[i] && sl.inner < kInnerCap) continue;
       // FP64 update: x += |r| e ; r = b - D x
       Spinor xi = ssub(x64, i, 1), ri = ssub(r64, i, 1);
-      MG_CHECK(convert_spinor(ctx, ssub(e32, i, 1), xi, s, dsc + cap + i, true));
+      if (even_odd) {
+        Spinor ei = ssub(e32, i, 1);
+        MG_CHECK(schur_odd_solution(ctx, G, &ei, ssub(ro, i, 1), to, s));
+        MG_CHECK(eo_join(ctx, G, ei, to, tf, xi, dsc + cap + i, s));
+      } else {
+        MG_CHECK(convert_spinor(ctx, ssub(e32, i, 1), xi, s, dsc + cap + i, true));
+      }
       MG_CHECK(dslash(ctx, G, xi, ri, false, false, s));  // r = D x, then r = b - r
       Vec rv = as_vec(ri);
       MG_CHECK(axpby(ctx, nullptr, C1, as_vec(ssub(b64, i, 1)), nullptr, CM1, rv, s));
