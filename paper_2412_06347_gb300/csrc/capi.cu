@@ -425,29 +425,10 @@ mglma_status mglma_dirac_apply(mglma_ctx ctx, mglma_gauge G, mglma_op op, int nr
     MG_CHECK(dirac_schur64(ctx, G, nrhs, sin.dev, sout.dev, op == MGLMA_OP_SCHUR_Q, s));
     return stage_out_finish(out, bytes, s, sout);
   }
-  Spinor a, b;
-  a.prec = b.prec = compute;
-  a.nrhs = b.nrhs = nrhs;
-  a.V = b.V = G->g.V;
-  mglma_status st = dalloc(ctx, &a.p, a.bytes(), s);
-  if (st == MGLMA_OK) st = dalloc(ctx, &b.p, b.bytes(), s);
-  if (st == MGLMA_OK) st = pack_spinor(ctx, sin.dev, a, s);
-  const Spinor* res = &b;
-  if (st == MGLMA_OK) {
-    switch (op) {
-      case MGLMA_OP_D: st = dslash(ctx, G, a, b, false, false, s); break;
-      case MGLMA_OP_DDAG: st = dslash(ctx, G, a, b, true, false, s); break;
-      case MGLMA_OP_Q: st = dslash(ctx, G, a, b, false, true, s); break;
-      case MGLMA_OP_DDAGD:
-        st = dslash(ctx, G, a, b, false, false, s);
-        if (st == MGLMA_OK) st = dslash(ctx, G, b, a, true, false, s);
-        res = &a;
-        break;
-    }
-  }
-  if (st == MGLMA_OK) st = unpack_spinor(ctx, *res, sout.dev, s);
-  dfree(ctx, a.p, s);
-  dfree(ctx, b.p, s);
+  void* work = nullptr;
+  mglma_status st = dalloc(ctx, &work, dirac_canonical_work(ctx, G, op, nrhs, compute, sin.dev, sout.dev), s);
+  if (st == MGLMA_OK) st = dirac_canonical(ctx, G, op, nrhs, sin.dev, sout.dev, compute, work, s);
+  dfree(ctx, work, s);
   if (st == MGLMA_OK) st = stage_out_finish(out, bytes, s, sout);
   return st;
 }

@@ -80,6 +80,9 @@ __global__ void __launch_bounds__(128, dslash_min_ctas<R, NR, RW>()) dslash_kern
   static_assert(!GD || (!RED && NR == 1 && RW == 1 && sizeof(R) == 4), "GCR dots: plain FP32 tile 1,1 only");
   static_assert(!RED || (NR == 1 && RW == 1 && sizeof(R) == 4), "fused reduction: FP32 tile 1,1 only");
   static_assert(!MRF || RED, "the fused MR step reduces its dots");
+  // FP32 result written as canonical complex128 (a warp stores together)
+  constexpr bool CAN = std::is_same<SO, Canon64>::value && sizeof(R) == 4;
+  static_assert(!CAN || (!RED && !GD && NR == 1 && RW == 1), "canonical output: plain FP32 tile 1,1 only");
   constexpr int SW = 128 / RW;  // sites per CTA
   const int64_t V = a.q.V;
   // RHS tile groups run fastest in launch order, so the CTAs that share a
@@ -91,7 +94,7 @@ __global__ void __launch_bounds__(128, dslash_min_ctas<R, NR, RW>()) dslash_kern
   if constexpr (RW == 1) {
     site = (int64_t)(blockIdx.x / ntile) * blockDim.x + threadIdx.x;
     if (site >= V) {
-      if constexpr (!RED && !GD) return;
+      if constexpr (!RED && !GD && !CAN) return;
       valid = false;
       site = V - 1;
     }
@@ -152,6 +155,17 @@ __global__ void __launch_bounds__(128, dslash_min_ctas<R, NR, RW>()) dslash_kern
           hop_add<R, false>(mu, sB, f, Um, psi, acc[r]);
         }
     }
+  }
+  if constexpr (CAN) {
+    __shared__ double2 sh[4][kCanonWarpDoubles2];
+    if (a.g5out) {
+#pragma unroll
+      for (int k = 6; k < 12; ++k) acc[0][k] = -acc[0][k];
+    }
+    const int64_t site0 = (int64_t)(blockIdx.x / ntile) * blockDim.x + (threadIdx.x & ~31u);
+    const int ns = (int)min((int64_t)32, V - site0);
+    store_canonical(sh[threadIdx.x / 32], reinterpret_cast<double2*>(out) + ((size_t)r0 * V + site0) * 12, ns, acc[0]);
+    return;
   }
   float nn = 0.f, dr = 0.f, di = 0.f;  // RED: this thread's |t|^2 and <t, s>
   constexpr bool BF = std::is_same<SO, SpinBf16>::value;
@@ -248,7 +262,7 @@ __global__ void __launch_bounds__(128, dslash_min_ctas<R, NR, RW>()) dslash_kern
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[r][k] = bf16_unpack(bf16_pack(acc[r][k]));
           }
-          SIO<SO>::store(out, V, r0 + r, site, acc[r]);
+          if constexpr (!CAN) SIO<SO>::store(out, V, r0 + r, site, acc[r]);
         }
       }
     if constexpr (RED) {
@@ -632,32 +646,184 @@ __global__ void __launch_bounds__(128) dslash_slot_kernel(const double2* __restr
   IO<double>::store(out, V, rhs, site, acc);
 }
 
+// ------------------------------------------------------------ FP64 stencil, four threads per site
+// Few sites: D (or D^dag) on canonical complex128 spinors, a CTA of four warps
+// per 32 sites of one RHS.  Warp mu takes the two hops of direction mu; the sums
+// meet in shared memory, and warp mu adds rows 3 mu .. 3 mu + 2 of the clover
+// term and writes those components.  With one thread per site an 8^4 spinor is
+// 128 warps, one per SM at most, each alone with its SM's FP64 pipe.
+template <bool DAG, int MU>
+__device__ __forceinline__ void split_hops(const double2* in, const double2* U, const DslashArgs& a, int r,
+                                           int64_t site, const int x[4], Cx<double> acc[12]) {
+  const double sF = DAG ? 1.0 : -1.0;
+  const int64_t V = a.q.V, nf = nbr_fwd(a.q, site, x, MU), nb = nbr_bwd(a.q, site, x, MU);
+  const double ff = -0.5 * ((MU == 0 && x[0] == a.q.L[0] - 1) ? a.bc : 1.0);
+  const double fb = -0.5 * ((MU == 0 && x[0] == 0) ? a.bc : 1.0);
+  Cx<double> psi[12];
+  M3<double> Um;
+  Link<double>::load(U, V, MU, site, Um);
+  SIO<Canon64>::load(in, V, r, nf, psi);
+  hop_add<double, true>(MU, sF, ff, Um, psi, acc);
+  Link<double>::load(U, V, MU, nb, Um);
+  SIO<Canon64>::load(in, V, r, nb, psi);
+  hop_add<double, false>(MU, -sF, fb, Um, psi, acc);
+}
+
+// o[k] += row 3 HALF + k of the packed Hermitian block times v
+template <int HALF>
+__device__ __forceinline__ void split_clover(const double c[36], const Cx<double> v[6], Cx<double> o[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int i = 3 * HALF + k;
+    Cx<double> s = c[i] * v[i];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      if (j == i) continue;
+      const int e = 6 + 2 * (i < j ? offdiag_slot(i, j) : offdiag_slot(j, i));
+      if (i < j)
+        cfma(s, cx(c[e], c[e + 1]), v[j]);
+      else
+        cfma_conj(s, cx(c[e], c[e + 1]), v[j]);
+    }
+    o[k] = o[k] + s;
+  }
+}
+
+template <bool DAG>
+__global__ void __launch_bounds__(128) dslash_split_kernel(const double2* __restrict__ in, double2* __restrict__ out,
+                                                           const double2* __restrict__ U, const double2* __restrict__ C,
+                                                           DslashArgs a) {
+  __shared__ double2 sh[4][12][32];
+  const int64_t V = a.q.V;
+  const int mu = threadIdx.x / 32, lane = threadIdx.x % 32, r = blockIdx.y;
+  const int64_t site0 = (int64_t)blockIdx.x * 32 + lane, site = site0 < V ? site0 : V - 1;
+  int x[4];
+  site_coords(a.q, site, x);
+  Cx<double> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = cx(0.0, 0.0);
+  switch (mu) {
+    case 0: split_hops<DAG, 0>(in, U, a, r, site, x, acc); break;
+    case 1: split_hops<DAG, 1>(in, U, a, r, site, x, acc); break;
+    case 2: split_hops<DAG, 2>(in, U, a, r, site, x, acc); break;
+    default: split_hops<DAG, 3>(in, U, a, r, site, x, acc); break;
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) sh[mu][k][lane] = make_double2(acc[k].re, acc[k].im);
+  const int chi = mu / 2;
+  double c[36];
+  Clover<double>::load(C, V, chi, site, c);
+  const double2* p = in + ((size_t)r * V + site) * 12 + 6 * chi;
+  Cx<double> v[6], o[3];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const double2 q = __ldg(p + k);
+    v[k] = cx(q.x, q.y);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    o[k] = cx(0.0, 0.0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const double2 q = sh[m][3 * mu + k][lane];
+      o[k] = o[k] + cx(q.x, q.y);
+    }
+  }
+  if (mu & 1)
+    split_clover<1>(c, v, o);
+  else
+    split_clover<0>(c, v, o);
+  if (site0 >= V) return;
+  const double g = a.g5out && chi ? -1.0 : 1.0;
+  double2* w = out + ((size_t)r * V + site) * 12 + 3 * mu;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) w[k] = make_double2(g * o[k].re, g * o[k].im);
+}
+
 // ------------------------------------------------------------ layout conversion
+// Canonical complex128 [rhs][site][12] <-> internal fields, a warp per 32 sites
+// of one RHS: the canonical side is read or written as whole rows of 512 bytes
+// and transposed through shared memory (one padding element per site keeps both
+// sides free of bank conflicts); FP32 is converted by integer arithmetic
+// (convert.cuh).  64x32^3, 16 RHS, FP32: 1.56 ms per pass (6.2 TB/s), 3.03 ms with
+// scattered 16-byte accesses and the FP64 pipe's conversions.
+constexpr int PK_WARPS = 4;
 template <typename R>
-__global__ void pack_kernel(const double* __restrict__ canon, void* __restrict__ dst, int64_t V, int nrhs) {
-  const int64_t site = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int r = blockIdx.y;
-  if (site >= V || r >= nrhs) return;
-  const double2* p = reinterpret_cast<const double2*>(canon) + ((size_t)r * V + site) * 12;
+struct Pk;
+template <>
+struct Pk<float> {
+  using E = float2;
+  static constexpr int S = 14;  // elements per site in shared memory (16-byte rows)
+  __device__ __forceinline__ static E from(double2 v) {
+    bool other = false;
+    E e = make_float2(d2f_fast(v.x, other), d2f_fast(v.y, other));
+    if (other) e = make_float2((float)v.x, (float)v.y);
+    return e;
+  }
+  __device__ __forceinline__ static double2 to(E v) {
+    bool other = false;
+    double2 d = make_double2(f2d_fast(v.x, other), f2d_fast(v.y, other));
+    if (other) d = make_double2((double)v.x, (double)v.y);
+    return d;
+  }
+};
+template <>
+struct Pk<double> {
+  using E = double2;
+  static constexpr int S = 13;
+  __device__ __forceinline__ static E from(double2 v) { return v; }
+  __device__ __forceinline__ static double2 to(E v) { return v; }
+};
+
+template <typename R>
+__global__ void __launch_bounds__(32 * PK_WARPS) pack_kernel(const double2* __restrict__ canon, void* __restrict__ dst,
+                                                             int64_t V) {
+  using P = Pk<R>;
+  __shared__ __align__(16) typename P::E sh[PK_WARPS][32 * P::S];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32, r = blockIdx.y;
+  const int64_t site0 = ((int64_t)blockIdx.x * PK_WARPS + w) * 32;
+  if (site0 >= V) return;
+  const int ns = (int)min((int64_t)32, V - site0);
+  const double2* p = canon + ((size_t)r * V + site0) * 12;
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    const int e = 32 * i + lane;
+    if (e < 12 * ns) sh[w][e / 12 * P::S + e % 12] = P::from(__ldg(p + e));
+  }
+  __syncwarp();
+  if (lane >= ns) return;
   Cx<R> s[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    double2 v = p[k];
-    s[k] = cx((R)v.x, (R)v.y);
-  }
-  IO<R>::store(dst, V, r, site, s);
+  for (int k = 0; k < 12; ++k) s[k] = cx(sh[w][lane * P::S + k].x, sh[w][lane * P::S + k].y);
+  IO<R>::store(dst, V, r, site0 + lane, s);
 }
 
 template <typename R>
-__global__ void unpack_kernel(const void* __restrict__ src, double* __restrict__ canon, int64_t V, int nrhs) {
-  const int64_t site = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int r = blockIdx.y;
-  if (site >= V || r >= nrhs) return;
-  Cx<R> s[12];
-  IO<R>::load(src, V, r, site, s);
-  double2* p = reinterpret_cast<double2*>(canon) + ((size_t)r * V + site) * 12;
+__global__ void __launch_bounds__(32 * PK_WARPS) unpack_kernel(const void* __restrict__ src, double2* __restrict__ canon,
+                                                               int64_t V) {
+  using P = Pk<R>;
+  __shared__ __align__(16) typename P::E sh[PK_WARPS][32 * P::S];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32, r = blockIdx.y;
+  const int64_t site0 = ((int64_t)blockIdx.x * PK_WARPS + w) * 32;
+  if (site0 >= V) return;
+  const int ns = (int)min((int64_t)32, V - site0);
+  if (lane < ns) {
+    Cx<R> s[12];
+    IO<R>::load(src, V, r, site0 + lane, s);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) p[k] = make_double2((double)s[k].re, (double)s[k].im);
+    for (int k = 0; k < 12; ++k) {
+      sh[w][lane * P::S + k].x = s[k].re;
+      sh[w][lane * P::S + k].y = s[k].im;
+    }
+  }
+  __syncwarp();
+  double2* p = canon + ((size_t)r * V + site0) * 12;
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    const int e = 32 * i + lane;
+    if (e < 12 * ns) p[e] = P::to(sh[w][e / 12 * P::S + e % 12]);
+  }
 }
 
 // dst = scale_r * src (+ dst if accumulate); scale NULL means 1
@@ -854,12 +1020,14 @@ static inline dim3 site_grid(int64_t V, int threads, int ny = 1) {
   return dim3((unsigned)((V + threads - 1) / threads), (unsigned)ny, 1);
 }
 
+static inline dim3 pk_grid(int64_t V, int nrhs) { return site_grid(V, 32 * PK_WARPS, nrhs); }
+
 mglma_status pack_spinor(mglma_ctx ctx, const double* canon, Spinor& dst, cudaStream_t s) {
   ProfScope ps(ctx, K_PACK, s);
   if (dst.prec == MGLMA_FP64)
-    pack_kernel<double><<<site_grid(dst.V, 256, dst.nrhs), 256, 0, s>>>(canon, dst.p, dst.V, dst.nrhs);
+    pack_kernel<double><<<pk_grid(dst.V, dst.nrhs), 32 * PK_WARPS, 0, s>>>((const double2*)canon, dst.p, dst.V);
   else
-    pack_kernel<float><<<site_grid(dst.V, 256, dst.nrhs), 256, 0, s>>>(canon, dst.p, dst.V, dst.nrhs);
+    pack_kernel<float><<<pk_grid(dst.V, dst.nrhs), 32 * PK_WARPS, 0, s>>>((const double2*)canon, dst.p, dst.V);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
@@ -867,9 +1035,9 @@ mglma_status pack_spinor(mglma_ctx ctx, const double* canon, Spinor& dst, cudaSt
 mglma_status unpack_spinor(mglma_ctx ctx, const Spinor& src, double* canon, cudaStream_t s) {
   ProfScope ps(ctx, K_PACK, s);
   if (src.prec == MGLMA_FP64)
-    unpack_kernel<double><<<site_grid(src.V, 256, src.nrhs), 256, 0, s>>>(src.p, canon, src.V, src.nrhs);
+    unpack_kernel<double><<<pk_grid(src.V, src.nrhs), 32 * PK_WARPS, 0, s>>>(src.p, (double2*)canon, src.V);
   else
-    unpack_kernel<float><<<site_grid(src.V, 256, src.nrhs), 256, 0, s>>>(src.p, canon, src.V, src.nrhs);
+    unpack_kernel<float><<<pk_grid(src.V, src.nrhs), 32 * PK_WARPS, 0, s>>>(src.p, (double2*)canon, src.V);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
@@ -899,6 +1067,12 @@ static double dslash_bytes(int64_t V, int nrhs, bool fp64) {
   return (double)V * (fp64 ? 1152.0 + 384.0 * nrhs : 480.0 + 192.0 * nrhs);
 }
 static double dslash_flops(int64_t V, int nrhs) { return 1896.0 * (double)V * nrhs; }
+
+// site-RHS products up to which the FP64 stencil on canonical fields takes four
+// threads per site: 4096 sites 16.6 against 43.4 us with one thread per site,
+// 16384 47.5 against 43.4 (one warp on each quarter of 128 SMs by then), 65536
+// the same
+constexpr size_t kSplitSites = 12288;
 
 template <typename R, int NR, int RW, typename SO = R>
 static void launch_dslash(const Spinor& in, Spinor& out, const void* U, const void* C, const DslashArgs& a,
@@ -989,6 +1163,103 @@ mglma_status dslash(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& in, Spi
   }
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
+}
+
+// FP64 on canonical spinors: four threads per site while that is what fills the
+// chip, see dslash_split_kernel
+static void launch_canon64(const mglma_gauge_s* G, const double* in, double* out, const DslashArgs& a, bool dagger,
+                           cudaStream_t s) {
+  if ((size_t)G->g.V * a.nrhs <= kSplitSites && a.nrhs <= 65535) {
+    const dim3 g((unsigned)((G->g.V + 31) / 32), (unsigned)a.nrhs, 1);
+    if (dagger)
+      dslash_split_kernel<true><<<g, 128, 0, s>>>((const double2*)in, (double2*)out, G->U64, G->C64, a);
+    else
+      dslash_split_kernel<false><<<g, 128, 0, s>>>((const double2*)in, (double2*)out, G->U64, G->C64, a);
+    return;
+  }
+  const size_t ctas = (size_t)((G->g.V + 127) / 128) * a.nrhs;
+  if (dagger)
+    dslash_kernel<double, 1, true, 1, false, false, Canon64, Canon64>
+        <<<(unsigned)ctas, 128, 0, s>>>(in, out, G->U64, G->C64, a);
+  else
+    dslash_kernel<double, 1, false, 1, false, false, Canon64, Canon64>
+        <<<(unsigned)ctas, 128, 0, s>>>(in, out, G->U64, G->C64, a);
+}
+
+// FP32: an internal field in, canonical complex128 out (64x32^3, 16 RHS: 3889 us
+// against 2930 + 1570 us for the stencil and an unpack pass)
+static void launch_canon32(const mglma_gauge_s* G, const Spinor& in, double* out, const DslashArgs& a, bool dagger,
+                           cudaStream_t s) {
+  const size_t ctas = (size_t)((G->g.V + 127) / 128) * a.nrhs;
+  if (dagger)
+    dslash_kernel<float, 1, true, 1, false, false, float, Canon64>
+        <<<(unsigned)ctas, 128, 0, s>>>(in.p, out, G->U32, G->C32, a);
+  else
+    dslash_kernel<float, 1, false, 1, false, false, float, Canon64>
+        <<<(unsigned)ctas, 128, 0, s>>>(in.p, out, G->U32, G->C32, a);
+}
+
+// whether two canonical batches share memory: the FP64 stencil then works on a
+// copy of its input (every other form has read all of in before it writes out)
+static bool overlap(const double* a, const double* b, size_t bytes) {
+  const char *p = (const char*)a, *q = (const char*)b;
+  return p < q + bytes && q < p + bytes;
+}
+
+size_t dirac_canonical_work(const mglma_ctx_s* ctx, const mglma_gauge_s* G, int op, int nrhs, int prec,
+                            const double* in, const double* out) {
+  const size_t field = (size_t)nrhs * G->g.V * 24 * (prec == MGLMA_FP64 ? 8 : 4);
+  if (prec == MGLMA_FP64) return op == MGLMA_OP_DDAGD || overlap(in, out, field) ? field : 0;
+  const bool fused = tuned(ctx, TUNE_DSLASH32_NR, nrhs, G->g.V, dslash32_default_tile(nrhs)) == dslash32_tile_code(1, 1);
+  return fused && op != MGLMA_OP_DDAGD ? field : (field + 255) / 256 * 256 + field;
+}
+
+mglma_status dirac_canonical(mglma_ctx ctx, const mglma_gauge_s* G, int op, int nrhs, const double* in, double* out,
+                             int prec, void* work, cudaStream_t s) {
+  DslashArgs a;
+  a.q = make_latidx(G->g.L);
+  a.bc = (double)G->g.t_bc;
+  a.nrhs = nrhs;
+  a.g5out = op == MGLMA_OP_Q ? 1 : 0;
+  const bool dag = op == MGLMA_OP_DDAG, two = op == MGLMA_OP_DDAGD;
+  const double flops = dslash_flops(G->g.V, nrhs);
+  if (prec == MGLMA_FP64) {
+    const double bytes = dslash_bytes(G->g.V, nrhs, true);
+    double* mid = two ? (double*)work : out;
+    const size_t field = (size_t)nrhs * G->g.V * 24 * sizeof(double);
+    if (!two && overlap(in, out, field)) {
+      MG_CUDA(cudaMemcpyAsync(work, in, field, cudaMemcpyDeviceToDevice, s));
+      in = (const double*)work;
+    }
+    {
+      ProfScope ps(ctx, K_DSLASH64, s, bytes, flops);
+      launch_canon64(G, in, mid, a, dag, s);
+    }
+    if (two) {
+      ProfScope ps(ctx, K_DSLASH64, s, bytes, flops);
+      launch_canon64(G, mid, out, a, true, s);
+    }
+    MG_LAUNCH_CHECK();
+    return MGLMA_OK;
+  }
+  Spinor x, y;
+  x.prec = y.prec = MGLMA_FP32;
+  x.nrhs = y.nrhs = nrhs;
+  x.V = y.V = G->g.V;
+  x.p = work;
+  y.p = (char*)work + (x.bytes() + 255) / 256 * 256;
+  MG_CHECK(pack_spinor(ctx, in, x, s));
+  if (two) MG_CHECK(dslash(ctx, G, x, y, false, false, s));
+  Spinor& last = two ? y : x;
+  if (tuned(ctx, TUNE_DSLASH32_NR, nrhs, G->g.V, dslash32_default_tile(nrhs)) == dslash32_tile_code(1, 1)) {
+    ProfScope ps(ctx, K_DSLASH32, s, dslash_bytes(G->g.V, nrhs, false) + 96.0 * (double)G->g.V * nrhs, flops);
+    launch_canon32(G, last, out, a, dag || two, s);
+    MG_LAUNCH_CHECK();
+    return MGLMA_OK;
+  }
+  Spinor& res = two ? x : y;
+  MG_CHECK(dslash(ctx, G, last, res, dag || two, a.g5out != 0, s));
+  return unpack_spinor(ctx, res, out, s);
 }
 
 // FP64 values split into double-float pairs, elementwise (two per float4)
@@ -1333,53 +1604,7 @@ extern "C" mglma_status mglma_dirac_apply_noalloc(mglma_ctx ctx, mglma_gauge G, 
   void* scratch = nullptr;
   MG_CHECK(noalloc_scratch(ctx->device, &scratch));
   cudaStream_t s = cuda_stream ? (cudaStream_t)cuda_stream : ctx->stream;
-  // Both work fields are fully overwritten (pack writes a, the stencil writes
-  // b), so nothing in the array needs clearing between calls.
-  Spinor a, b;
-  a.prec = b.prec = compute;
-  a.nrhs = b.nrhs = nrhs;
-  a.V = b.V = G->g.V;
-  a.p = scratch;
-  b.p = static_cast<unsigned char*>(scratch) + ((field + 255) / 256) * 256;
-  DslashArgs da;
-  da.q = make_latidx(G->g.L);
-  da.bc = (double)G->g.t_bc;
-  da.nrhs = nrhs;
-  da.g5out = op == MGLMA_OP_Q ? 1 : 0;
-  const dim3 pg = site_grid(G->g.V, 256, nrhs);
-  const bool dp = compute == MGLMA_FP64;
-  const int kd = dp ? K_DSLASH64 : K_DSLASH32;
-  {
-    ProfScope ps(ctx, K_PACK, s);
-    if (dp)
-      pack_kernel<double><<<pg, 256, 0, s>>>(in, a.p, a.V, nrhs);
-    else
-      pack_kernel<float><<<pg, 256, 0, s>>>(in, a.p, a.V, nrhs);
-  }
-  const bool dag1 = op == MGLMA_OP_DDAG;
-  {
-    ProfScope ps(ctx, kd, s, dslash_bytes(G->g.V, nrhs, dp), dslash_flops(G->g.V, nrhs));
-    if (dp)
-      launch_dslash<double, 1, 1>(a, b, G->U64, G->C64, da, dag1, s);
-    else
-      launch_dslash<float, 1, 1>(a, b, G->U32, G->C32, da, dag1, s);
-  }
-  const Spinor* res = &b;
-  if (op == MGLMA_OP_DDAGD) {  // second pass D^dag back into a
-    ProfScope ps(ctx, kd, s, dslash_bytes(G->g.V, nrhs, dp), dslash_flops(G->g.V, nrhs));
-    if (dp)
-      launch_dslash<double, 1, 1>(b, a, G->U64, G->C64, da, true, s);
-    else
-      launch_dslash<float, 1, 1>(b, a, G->U32, G->C32, da, true, s);
-    res = &a;
-  }
-  {
-    ProfScope ps(ctx, K_PACK, s);
-    if (dp)
-      unpack_kernel<double><<<pg, 256, 0, s>>>(res->p, out, res->V, nrhs);
-    else
-      unpack_kernel<float><<<pg, 256, 0, s>>>(res->p, out, res->V, nrhs);
-  }
-  MG_LAUNCH_CHECK();
-  return MGLMA_OK;
+  // The work fields are fully overwritten before they are read, so nothing in
+  // the array needs clearing between calls.
+  return dirac_canonical(ctx, G, op, nrhs, in, out, compute, scratch, s);
 }

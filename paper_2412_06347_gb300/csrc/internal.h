@@ -278,6 +278,12 @@ mglma_status convert_spinor(mglma_ctx, const Spinor& src, Spinor& dst, cudaStrea
 // fine operator application: out = op(in), op in {D, D^dag, gamma5 D, gamma5 D^dag}
 mglma_status dslash(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, Spinor& out, bool dagger,
                     bool gamma5_out, cudaStream_t s);
+// out = op(in) on canonical device fields (D, D^dag, gamma5 D, D^dag D; out may be
+// in), with dirac_canonical_work bytes of work memory (16-byte aligned)
+size_t dirac_canonical_work(const mglma_ctx_s*, const mglma_gauge_s* G, int op, int nrhs, int prec, const double* in,
+                            const double* out);
+mglma_status dirac_canonical(mglma_ctx, const mglma_gauge_s* G, int op, int nrhs, const double* in, double* out,
+                             int prec, void* work, cudaStream_t s);
 // One fused MR smoothing step (the (1,1) stencil tile; t, tn, sk FP32 or all
 // BF16, z FP32): with u = D t,
 // tn = t - alpha u, sk <- sk - alpha t, z <- z + alpha sk (alpha per RHS, the

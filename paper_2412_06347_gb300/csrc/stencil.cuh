@@ -10,6 +10,7 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "convert.cuh"
 #include "cplx.cuh"
 #include "df.cuh"
 #include "internal.h"
@@ -125,6 +126,29 @@ struct SIO<SpinF32Df> {
     IO<float>::load(b, V, rhs, site, f);
 #pragma unroll
     for (int k = 0; k < 12; ++k) s[k] = cx(DF(f[k].re, 0.f), DF(f[k].im, 0.f));
+  }
+};
+// canonical complex128 spinors ([rhs][site][12]) read or written in place of an
+// internal field.  FP64: the stencil is bound by the FP64 pipe (1130
+// instructions per site at about 2 lanes per clock and SM), so its scattered
+// 16-byte accesses (each thread walks its site's 192 bytes) cost nothing and
+// save both layout passes.  FP32: output only, see store_canonical.
+struct Canon64 {};
+template <>
+struct SIO<Canon64> {
+  using R = double;
+  __device__ __forceinline__ static void load(const void* b, int64_t V, int rhs, int64_t site, Cx<double> s[12]) {
+    const double2* p = reinterpret_cast<const double2*>(b) + ((size_t)rhs * V + site) * 12;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 v = __ldg(p + k);
+      s[k] = cx(v.x, v.y);
+    }
+  }
+  __device__ __forceinline__ static void store(void* b, int64_t V, int rhs, int64_t site, const Cx<double> s[12]) {
+    double2* p = reinterpret_cast<double2*>(b) + ((size_t)rhs * V + site) * 12;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) p[k] = make_double2(s[k].re, s[k].im);
   }
 };
 // output of the double-float residual update: out (FP64 spinors) -=
@@ -355,6 +379,35 @@ __device__ __forceinline__ void hop_add(int mu, R s, R f, const M3<R>& U, const 
     g1[c] = f * g1[c];
   }
   reconstruct_add<R>(mu, s, g0, g1, acc);
+}
+
+// a warp's 32 consecutive sites site0.. (ns of them exist) of one RHS, FP32 in
+// registers (lane = site), to canonical complex128: through shared memory in two
+// halves of six components (padded to seven, so both sides are free of bank
+// conflicts), so the warp writes whole sectors
+constexpr int kCanonWarpDoubles2 = 32 * 7;
+__device__ __forceinline__ void store_canonical(double2* sh, double2* dst, int ns, const Cx<float> s[12]) {
+  const int lane = threadIdx.x % 32;
+  bool other = false;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    double2 d[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      d[k] = make_double2(f2d_fast(s[6 * half + k].re, other), f2d_fast(s[6 * half + k].im, other));
+    if (other)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) d[k] = make_double2((double)s[6 * half + k].re, (double)s[6 * half + k].im);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sh[lane * 7 + k] = d[k];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const int e = 32 * i + lane, x = e / 6, k = e % 6;
+      if (x < ns) dst[(size_t)x * 12 + 6 * half + k] = sh[x * 7 + k];
+    }
+  }
 }
 
 struct DslashArgs {
