@@ -7,8 +7,6 @@
 // then FP64) in a fixed two-stage order, so results are bitwise reproducible
 // and independent of how RHS are grouped.
 #include "internal.h"
-#include "minres.cuh"
-
 
 namespace mglma {
 
@@ -405,8 +403,6 @@ __device__ __forceinline__ double2 rscale(double2 x, double a) { return make_dou
 
 // Lanczos step z -= a_r v + b_r u with a_r = Re dot[r], b_r = beta[r], and
 // out1[r] = |z_r|^2; RHS with active[r] == 0 are left alone (out1 = 0).
-// With st, the last block of each RHS then runs that RHS's MINRES scalar
-// step (minres.cuh; out1 must be its MR_BN2 slot).
 template <typename R>
 __global__ void __launch_bounds__(RT) lanczos_norm_kernel(const typename Pair<R>::T* __restrict__ v,
                                                           const typename Pair<R>::T* __restrict__ u,
@@ -415,8 +411,7 @@ __global__ void __launch_bounds__(RT) lanczos_norm_kernel(const typename Pair<R>
                                                           const double* __restrict__ beta,
                                                           const int* active, size_t m,
                                                           double2* __restrict__ part, unsigned* __restrict__ count,
-                                                          double* out1, double* st, double tol, int cap,
-                                                          int* act) {
+                                                          double* out1) {
   const int r = blockIdx.y, nrhs = gridDim.y, nb = gridDim.x;
   const bool on = active[r] != 0;
   const double a = on ? -dot[r].x : 0.0, b = on ? -beta[r] : 0.0;
@@ -431,8 +426,7 @@ __global__ void __launch_bounds__(RT) lanczos_norm_kernel(const typename Pair<R>
   }
   const double2 t = block_sum2<RT>(make_double2(acc.norm(), 0));
   if (threadIdx.x == 0) part[(size_t)r * nb + blockIdx.x] = t;
-  if (finish<0>(part, count, 1, nb, nrhs, nullptr, out1) && st && threadIdx.x == 0)
-    minres_scalar_step(st, dot, act, tol, cap, r);
+  finish<0>(part, count, 1, nb, nrhs, nullptr, out1);
 }
 
 // w_new = cf0 v + cf1 w1 + cf2 w2 ; x += cf3 w_new ; z *= cf4, for RHS with
@@ -589,6 +583,10 @@ static mglma_status red_scratch(mglma_ctx ctx, cudaStream_t s, size_t nparts, in
   return MGLMA_OK;
 }
 
+mglma_status red_buffers(mglma_ctx ctx, cudaStream_t s, size_t nparts, int ncount, double2** part, unsigned** count) {
+  return red_scratch(ctx, s, nparts, ncount, part, count);
+}
+
 mglma_status red_scratch_ready(mglma_ctx ctx, cudaStream_t s) {
   double2* p;
   unsigned* c;
@@ -708,8 +706,8 @@ mglma_status axpy2_norm(mglma_ctx ctx, const double2* a, const Vec& p, Vec& x, c
   return MGLMA_OK;
 }
 
-mglma_status lanczos_norm(mglma_ctx ctx, const double2* dot, const double* beta, int* active, const Vec& v,
-                          const Vec& u, Vec& z, double* zz, cudaStream_t s, double* st, double tol, int cap) {
+mglma_status lanczos_norm(mglma_ctx ctx, const double2* dot, const double* beta, const int* active, const Vec& v,
+                          const Vec& u, Vec& z, double* zz, cudaStream_t s) {
   if (v.prec != z.prec || u.prec != z.prec || v.n != z.n || u.n != z.n)
     return fail(MGLMA_ERR_INVALID, "lanczos_norm: mismatch");
   if (z.nrhs == 0) return MGLMA_OK;
@@ -722,10 +720,10 @@ mglma_status lanczos_norm(mglma_ctx ctx, const double2* dot, const double* beta,
   dim3 g(nb, z.nrhs, 1);
   if (z.prec == MGLMA_FP64)
     lanczos_norm_kernel<double><<<g, RT, 0, s>>>((const double2*)v.p, (const double2*)u.p, (double2*)z.p, dot, beta,
-                                                 active, m, part, count, zz, st, tol, cap, active);
+                                                 active, m, part, count, zz);
   else
     lanczos_norm_kernel<float><<<g, RT, 0, s>>>((const float4*)v.p, (const float4*)u.p, (float4*)z.p, dot, beta,
-                                                active, m, part, count, zz, st, tol, cap, active);
+                                                active, m, part, count, zz);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }

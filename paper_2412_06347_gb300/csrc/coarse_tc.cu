@@ -33,6 +33,7 @@
 
 #include "internal.h"
 #include "lattice.cuh"
+#include "minres.cuh"
 #include "tcgen05.cuh"
 #include "solver.h"
 #include "subspace.h"
@@ -103,44 +104,132 @@ __global__ void x_image_kernel(const float2* __restrict__ X, uint4* __restrict__
   x_image_store(XB + ((size_t)t * V1 + z) * rows, jo, G, NT, ri, re, im);
 }
 
-// The coarse MINRES update (w_new = cf0 v + cf1 w1 + cf2 w2, x += cf3 w_new,
-// z *= cf4 for RHS with cf5 != 0; cf_j[r] = cf[j stride + r]) on FP32
-// half-lattice fields, which also writes the B-operand image (tiles of NT,
-// no gamma5hat) of the scaled z -- the next iteration's Lanczos vector -- so
-// its operator application needs no image pass.  One thread per (site, group
-// of 8 dofs) of RHS blockIdx.y.
-__global__ void minres_update_image_kernel(const float4* __restrict__ v, const float4* __restrict__ w1,
-                                           const float4* __restrict__ w2, float4* __restrict__ wn,
-                                           float4* __restrict__ x, float4* __restrict__ z,
-                                           const double* __restrict__ cf, int stride, int64_t Vh, int n2, int NT,
-                                           uint4* __restrict__ XB) {
-  const int r = blockIdx.y;
-  if (cf[5 * (size_t)stride + r] == 0.0) return;
-  const float c0 = (float)cf[r], c1 = (float)cf[stride + r], c2 = (float)cf[2 * (size_t)stride + r],
-              c3 = (float)cf[3 * (size_t)stride + r], c4 = (float)cf[4 * (size_t)stride + r];
+// One coarse MINRES iteration after the operator (Y_k = Q u_k and dot = <u_k, Y_k>
+// from the tensor-core launches) on FP32 half-lattice fields, for unnormalised
+// Lanczos vectors (minres.cuh): with the coefficients of its RHS blockIdx.y,
+//   Y <- u_(k+1) = c1 Y + c2 u_k + c3 u_(k-1), its B-operand image (tiles of NT,
+//   no gamma5hat) for the next operator application, |u_(k+1)|^2, and
+//   the pending update of iteration k - 1: w_(k-1) = cf0 u_(k-1) + cf1 w_(k-2)
+//   + cf2 w_(k-3) (into w_(k-3)'s place), x += cf3 w_(k-1);
+// the last block of the RHS adds the partial norms in order and runs the scalar
+// step, which leaves iteration k's update pending.  Traffic and latency bound:
+// ten field passes per iteration in one launch, against thirteen in two launches
+// with normalised vectors (the scaled vector and its image needed the norm
+// first).  One thread per (site, group of 8 dofs); the blocks of a RHS depend on
+// the volume alone.
+struct LanczosRun {
+  const float4 *u, *uo, *w1;
+  float4 *y, *w2, *x;
+  double* st;
+  const double2* dot;
+  int* active;
+  double tol;
+  int cap;
+  double* part;  // [nrhs][blocks of a RHS]
+  unsigned* count;
+};
+constexpr int LZ_T = 128;
+__global__ void __launch_bounds__(LZ_T) lanczos_step_kernel(LanczosRun run, int64_t Vh, int n2, int NT,
+                                                            uint4* __restrict__ XB) {
+  const int r = blockIdx.y, nb = gridDim.x;
+  __shared__ float cs[7];
+  __shared__ int flags[2];
+  if (threadIdx.x == 0) {
+    auto S = [&](int j) { return run.st[(size_t)j * run.cap + r]; };
+    flags[0] = run.active[r];
+    flags[1] = S(MR_CF + 5) != 0.0;
+    cs[0] = (float)S(MR_LC);
+    cs[1] = (float)(run.dot[r].x * S(MR_LC + 1));
+    cs[2] = (float)S(MR_LC + 2);
+    for (int j = 0; j < 4; ++j) cs[3 + j] = (float)S(MR_CF + j);
+  }
+  __syncthreads();
+  const bool on = flags[0] != 0, pend = flags[1] != 0;
+  if (!on && !pend) return;
+  const float c1 = cs[0], c2 = cs[1], c3 = cs[2], f0 = cs[3], f1 = cs[4], f2 = cs[5], f3 = cs[6];
   const int G = n2 / 8;
   const size_t ng = (size_t)Vh * G, off = (size_t)r * Vh * (n2 / 2);
   const size_t rows = (size_t)2 * G * 2 * NT;
-  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += (size_t)gridDim.x * blockDim.x) {
-    float re[8], im[8];
+  double N = 0;
+  for (size_t g = (size_t)blockIdx.x * LZ_T + threadIdx.x; g < ng; g += (size_t)nb * LZ_T) {
+    const size_t i0 = off + 4 * g;
+    float4 b[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const size_t i = off + 4 * g + q;
-      const float4 a = v[i], b = w1[i], c = w2[i];
-      const float4 w = make_float4(c0 * a.x + c1 * b.x + c2 * c.x, c0 * a.y + c1 * b.y + c2 * c.y,
-                                   c0 * a.z + c1 * b.z + c2 * c.z, c0 * a.w + c1 * b.w + c2 * c.w);
-      wn[i] = w;
-      const float4 xo = x[i];
-      x[i] = make_float4(xo.x + c3 * w.x, xo.y + c3 * w.y, xo.z + c3 * w.z, xo.w + c3 * w.w);
-      const float4 zo = z[i];
-      const float4 zn = make_float4(c4 * zo.x, c4 * zo.y, c4 * zo.z, c4 * zo.w);
-      z[i] = zn;
-      re[2 * q] = zn.x;
-      im[2 * q] = zn.y;
-      re[2 * q + 1] = zn.z;
-      im[2 * q + 1] = zn.w;
+    for (int q = 0; q < 4; ++q) b[q] = run.uo[i0 + q];
+    if (on) {
+      float re[8], im[8], n = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 y = run.y[i0 + q], a = run.u[i0 + q];
+        const float4 z = make_float4(c1 * y.x + c2 * a.x + c3 * b[q].x, c1 * y.y + c2 * a.y + c3 * b[q].y,
+                                     c1 * y.z + c2 * a.z + c3 * b[q].z, c1 * y.w + c2 * a.w + c3 * b[q].w);
+        run.y[i0 + q] = z;
+        n += z.x * z.x + z.y * z.y + z.z * z.z + z.w * z.w;
+        re[2 * q] = z.x;
+        im[2 * q] = z.y;
+        re[2 * q + 1] = z.z;
+        im[2 * q + 1] = z.w;
+      }
+      N += (double)n;
+      x_image_store(XB + ((size_t)(r / NT) * Vh + (int64_t)(g / G)) * rows, (int)(g % G), G, NT, r % NT, re, im);
     }
-    x_image_store(XB + ((size_t)(r / NT) * Vh + (int64_t)(g / G)) * rows, (int)(g % G), G, NT, r % NT, re, im);
+    if (pend) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 c = run.w1[i0 + q], d = run.w2[i0 + q], xo = run.x[i0 + q];
+        const float4 w = make_float4(f0 * b[q].x + f1 * c.x + f2 * d.x, f0 * b[q].y + f1 * c.y + f2 * d.y,
+                                     f0 * b[q].z + f1 * c.z + f2 * d.z, f0 * b[q].w + f1 * c.w + f2 * d.w);
+        run.w2[i0 + q] = w;
+        run.x[i0 + q] = make_float4(xo.x + f3 * w.x, xo.y + f3 * w.y, xo.z + f3 * w.z, xo.w + f3 * w.w);
+      }
+    }
+  }
+  auto block_sum = [&](double v) -> double {  // valid in thread 0
+    __shared__ double sh[LZ_T / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (threadIdx.x % 32 == 0) sh[threadIdx.x / 32] = v;
+    __syncthreads();
+    v = 0;
+    if (threadIdx.x == 0)
+      for (int w = 0; w < LZ_T / 32; ++w) v += sh[w];
+    return v;
+  };
+  const double t = block_sum(N);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    run.part[(size_t)r * nb + blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(run.count + r, 1u) == (unsigned)(nb - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double a = 0;
+  for (int i = threadIdx.x; i < nb; i += LZ_T) a += __ldcg(run.part + (size_t)r * nb + i);
+  a = block_sum(a);
+  if (threadIdx.x == 0) {
+    run.count[r] = 0;
+    run.st[(size_t)MR_BN2 * run.cap + r] = a;
+    minres_scalar_step_u(run.st, run.dot[r].x, run.active, run.tol, run.cap, r);
+  }
+}
+
+// the update the last lanczos_step_kernel left pending (x only): x += cf3 (cf0 u
+// + cf1 w1 + cf2 w2)
+__global__ void minres_flush_kernel(const float4* __restrict__ u, const float4* __restrict__ w1,
+                                    const float4* __restrict__ w2, float4* __restrict__ x,
+                                    const double* __restrict__ cf, int cap, size_t m) {
+  const int r = blockIdx.y;
+  if (cf[5 * (size_t)cap + r] == 0.0) return;
+  const float f3 = (float)cf[3 * (size_t)cap + r], f0 = (float)cf[r], f1 = (float)cf[cap + r],
+              f2 = (float)cf[2 * (size_t)cap + r];
+  const size_t off = (size_t)r * m;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 b = u[off + i], c = w1[off + i], d = w2[off + i], xo = x[off + i];
+    x[off + i] = make_float4(xo.x + f3 * (f0 * b.x + f1 * c.x + f2 * d.x), xo.y + f3 * (f0 * b.y + f1 * c.y + f2 * d.y),
+                             xo.z + f3 * (f0 * b.z + f1 * c.z + f2 * d.z), xo.w + f3 * (f0 * b.w + f1 * c.w + f2 * d.w));
   }
 }
 
@@ -681,22 +770,49 @@ mglma_status coarse_x_image_half(mglma_ctx ctx, const mglma_coarse_s* C, const v
   return MGLMA_OK;
 }
 
-mglma_status minres_update_image(mglma_ctx ctx, const mglma_coarse_s* C, const double* cf, int stride, const Vec& v,
-                                 const Vec& w1, const Vec& w2, Vec& wn, Vec& x, Vec& z, void* image, cudaStream_t s) {
+mglma_status lanczos_step(mglma_ctx ctx, const mglma_coarse_s* C, double* st, int cap, const double2* dot, int* active,
+                          double tol, const Vec& u, const Vec& uo, Vec& y, const Vec& w1, Vec& w2, Vec& x, void* image,
+                          cudaStream_t s) {
   const int n2 = C->n2;
   const int64_t Vh = C->geo.V1 / 2;
-  if (x.prec != MGLMA_FP32 || n2 % 8 || x.n != (size_t)Vh * n2 * 2 || v.n != x.n || w1.n != x.n || w2.n != x.n ||
-      wn.n != x.n || z.n != x.n)
-    return fail(MGLMA_ERR_INVALID, "minres_update_image: FP32 half-lattice fields needed");
+  for (const Vec* v : {&u, &uo, (const Vec*)&y, &w1, (const Vec*)&w2, (const Vec*)&x})
+    if (v->prec != MGLMA_FP32 || v->n != (size_t)Vh * n2 * 2 || v->nrhs != x.nrhs || n2 % 8)
+      return fail(MGLMA_ERR_INVALID, "lanczos_step: FP32 half-lattice fields needed");
   if (x.nrhs == 0) return MGLMA_OK;
   const int NT = coarse_tc_nt(ctx, C, x.nrhs);
-  ProfScope ps(ctx, K_BLAS, s, 8.0 * x.bytes() + (double)x.nrhs * Vh * n2 * 8.0);
   const size_t ng = (size_t)Vh * (n2 / 8);
-  const unsigned gx = (unsigned)std::min<size_t>((ng + 255) / 256, std::max(4, 8 * ctx->sm_count / x.nrhs + 1));
-  dim3 g(gx, x.nrhs, 1);
-  minres_update_image_kernel<<<g, 256, 0, s>>>((const float4*)v.p, (const float4*)w1.p, (const float4*)w2.p,
-                                               (float4*)wn.p, (float4*)x.p, (float4*)z.p, cf, stride, Vh, n2, NT,
-                                               (uint4*)image);
+  const int nb = (int)std::min<size_t>((ng + LZ_T - 1) / LZ_T, 192);
+  double2* part = nullptr;
+  unsigned* count = nullptr;
+  MG_CHECK(red_buffers(ctx, s, (size_t)nb * x.nrhs, x.nrhs, &part, &count));
+  LanczosRun run;
+  run.u = (const float4*)u.p;
+  run.uo = (const float4*)uo.p;
+  run.w1 = (const float4*)w1.p;
+  run.y = (float4*)y.p;
+  run.w2 = (float4*)w2.p;
+  run.x = (float4*)x.p;
+  run.st = st;
+  run.dot = dot;
+  run.active = active;
+  run.tol = tol;
+  run.cap = cap;
+  run.part = (double*)part;
+  run.count = count;
+  ProfScope ps(ctx, K_BLAS, s, 10.0 * x.bytes());
+  lanczos_step_kernel<<<dim3((unsigned)nb, (unsigned)x.nrhs), LZ_T, 0, s>>>(run, Vh, n2, NT, (uint4*)image);
+  MG_LAUNCH_CHECK();
+  return MGLMA_OK;
+}
+
+mglma_status minres_flush(mglma_ctx ctx, const double* cf, int cap, const Vec& u, const Vec& w1, const Vec& w2, Vec& x,
+                          cudaStream_t s) {
+  if (x.nrhs == 0) return MGLMA_OK;
+  ProfScope ps(ctx, K_BLAS, s, 5.0 * x.bytes());
+  const size_t m = x.n / 4;
+  const unsigned gx = (unsigned)std::min<size_t>((m + 255) / 256, 128);
+  minres_flush_kernel<<<dim3(gx, (unsigned)x.nrhs), 256, 0, s>>>((const float4*)u.p, (const float4*)w1.p,
+                                                                 (const float4*)w2.p, (float4*)x.p, cf, cap, m);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }

@@ -422,6 +422,9 @@ mglma_status multi_cdot(mglma_ctx, const Vec& x0, size_t jstride_reals, int k, c
                         cudaStream_t s);
 // out[r] = |x_r|^2
 mglma_status norm2(mglma_ctx, const Vec& x, double* out, cudaStream_t s);
+// the stream's reduction scratch: nparts double2 partials and ncount tickets that
+// are zero before and after every reduction
+mglma_status red_buffers(mglma_ctx, cudaStream_t s, size_t nparts, int ncount, double2** part, unsigned** count);
 // allocates the stream's reduction scratch (must happen before a graph capture)
 mglma_status red_scratch_ready(mglma_ctx, cudaStream_t s);
 // accumulates the launch times of a replayed graph's event brackets
@@ -433,11 +436,8 @@ mglma_status axpy2_norm(mglma_ctx, const double2* a, const Vec& p, Vec& x, const
                         cudaStream_t s);
 // MINRES: z -= Re(dot_r) v + beta_r u, zz[r] = |z_r|^2 (RHS with active[r] == 0
 // are left alone, zz = 0)
-// st (nullable): also runs the MINRES scalar step of each RHS (minres.cuh)
-// in the kernel's last block; zz must then be st's MR_BN2 slot
-mglma_status lanczos_norm(mglma_ctx, const double2* dot, const double* beta, int* active, const Vec& v,
-                          const Vec& u, Vec& z, double* zz, cudaStream_t s, double* st = nullptr, double tol = 0,
-                          int cap = 0);
+mglma_status lanczos_norm(mglma_ctx, const double2* dot, const double* beta, const int* active, const Vec& v,
+                          const Vec& u, Vec& z, double* zz, cudaStream_t s);
 // MINRES: wn = c0 v + c1 w1 + c2 w2 ; x += c3 wn ; z *= c4 for RHS with c5 != 0,
 // c_j[r] = cf[j * stride + r] (real, device)
 mglma_status minres_update(mglma_ctx, const double* cf, int stride, const Vec& v, const Vec& w1, const Vec& w2,

@@ -388,6 +388,10 @@ __global__ void minres_init_kernel(double* st, int* active, int cap, int n) {
   S(MR_C2) = S(MR_C1) = 1;
   S(MR_S2) = S(MR_S1) = 0;
   S(MR_CF + 4) = on ? 1.0 / b1 : 0.0;
+  S(MR_CF + 5) = 0;  // no update pending
+  S(MR_LC) = 1;      // u_0 = v_0
+  S(MR_LC + 1) = -1;
+  S(MR_LC + 2) = 0;
   active[r] = on ? 1 : 0;
 }
 
@@ -431,11 +435,13 @@ struct MinresWork {
 
 static mglma_status minres_init(MinresWork& w, const mglma_coarse_s* C, const Vec& b, Vec& x) {
   const int n = b.nrhs;
-  Vec v0 = w.view(w.Vp, 0, n), vm = w.view(w.Vp, 2, n), w1 = w.view(w.Wp, 1, n), w2 = w.view(w.Wp, 2, n);
+  Vec v0 = w.view(w.Vp, 0, n), vm = w.view(w.Vp, 2, n);
   MG_CHECK(zero_vec(w.ctx, x, w.s));
   MG_CHECK(zero_vec(w.ctx, vm, w.s));
-  MG_CHECK(zero_vec(w.ctx, w1, w.s));
-  MG_CHECK(zero_vec(w.ctx, w2, w.s));
+  for (int j = 0; j < 3; ++j) {
+    Vec wj = w.view(w.Wp, j, n);
+    MG_CHECK(zero_vec(w.ctx, wj, w.s));
+  }
   MG_CHECK(norm2(w.ctx, b, w.st(MR_BB), w.s));
   {
     ProfScope ps(w.ctx, K_SCALAR, w.s);
@@ -446,27 +452,29 @@ static mglma_status minres_init(MinresWork& w, const mglma_coarse_s* C, const Ve
 }
 
 // eo: the vectors hold the even sites only and the operator is g5hat S_ee
-// (even-odd preconditioning, coarse_eo.cu), else all sites and g5hat D1
+// (even-odd preconditioning, coarse_eo.cu), else all sites and g5hat D1.
+// Where the last tensor-core launch can take the dot in its epilogue the
+// iteration runs on unnormalised Lanczos vectors in three launches (the
+// operator's input image is the previous step's, or the initialisation's) and
+// its update stays pending until the next one or minres_end; w_k sits in
+// direction slot k mod 2.
+static bool minres_unnormalised(const MinresWork& w, const mglma_coarse_s* C, int n, bool eo) {
+  return eo && coarse_schur_dot_ok(w.ctx, C, n, MGLMA_FP32);
+}
 static mglma_status minres_iter(MinresWork& w, const mglma_coarse_s* C, Vec& x, int n, int k, double tol,
                                 void* scr, size_t scr_bytes, bool eo = false) {
   const int a = k % 3, b = (k + 1) % 3, c = (k + 2) % 3;
   Vec v = w.view(w.Vp, a, n), vo = w.view(w.Vp, c, n), z = w.view(w.Vp, b, n);
+  if (minres_unnormalised(w, C, n, eo)) {
+    Vec w1 = w.view(w.Wp, k % 2, n), w2 = w.view(w.Wp, (k + 1) % 2, n);  // w_(k-2), w_(k-3)
+    MG_CHECK(coarse_schur_apply(w.ctx, C, v.p, z.p, n, MGLMA_FP32, CMODE_Q, scr, scr_bytes, w.s, w.sc.z, true));
+    return lanczos_step(w.ctx, C, w.sc.d, w.cap, w.sc.z, w.sc.active, tol, v, vo, z, w1, w2, x, scr, w.s);
+  }
   Vec wn = w.view(w.Wp, a, n), w1 = w.view(w.Wp, c, n), w2 = w.view(w.Wp, b, n);
-  // alpha = <v, Qhat v>: in the last tensor-core launch's epilogue when it
-  // can; then the operator's input image of v was written by the previous
-  // update (or by the initialisation), the scalar step runs at the end of the
-  // Lanczos-norm kernel, and the update writes the image of the next v
-  const bool fused_dot = eo && coarse_schur_dot_ok(w.ctx, C, n, MGLMA_FP32);
   if (eo)
-    MG_CHECK(coarse_schur_apply(w.ctx, C, v.p, z.p, n, MGLMA_FP32, CMODE_Q, scr, scr_bytes, w.s,
-                                fused_dot ? w.sc.z : nullptr, fused_dot));
+    MG_CHECK(coarse_schur_apply(w.ctx, C, v.p, z.p, n, MGLMA_FP32, CMODE_Q, scr, scr_bytes, w.s));
   else
     MG_CHECK(coarse_apply(w.ctx, C, v.p, z.p, n, MGLMA_FP32, CMODE_Q, w.s, scr, scr_bytes));
-  if (fused_dot) {
-    MG_CHECK(lanczos_norm(w.ctx, w.sc.z, w.st(MR_BETA), w.sc.active, v, vo, z, w.st(MR_BN2), w.s, w.sc.d, tol,
-                          w.cap));
-    return minres_update_image(w.ctx, C, w.st(MR_CF), w.cap, v, w1, w2, wn, x, z, scr, w.s);
-  }
   MG_CHECK(cdot(w.ctx, v, z, w.sc.z, w.s));
   MG_CHECK(lanczos_norm(w.ctx, w.sc.z, w.st(MR_BETA), w.sc.active, v, vo, z, w.st(MR_BN2), w.s));
   {
@@ -475,6 +483,13 @@ static mglma_status minres_iter(MinresWork& w, const mglma_coarse_s* C, Vec& x, 
     MG_LAUNCH_CHECK();
   }
   return minres_update(w.ctx, w.st(MR_CF), w.cap, v, w1, w2, wn, x, z, w.s);
+}
+
+// x after `iters` iterations, iters a multiple of 6: the pending update of the
+// last one (vector slot 2, w_(k-1) in direction slot 0, w_(k-2) in slot 1)
+static mglma_status minres_end(MinresWork& w, const mglma_coarse_s* C, Vec& x, int n, bool eo) {
+  if (!minres_unnormalised(w, C, n, eo)) return MGLMA_OK;
+  return minres_flush(w.ctx, w.st(MR_CF), w.cap, w.view(w.Vp, 2, n), w.view(w.Wp, 0, n), w.view(w.Wp, 1, n), x, w.s);
 }
 
 static mglma_status read_mask(const int* dev, int n, std::vector<int>& h, cudaStream_t s) {
@@ -678,9 +693,13 @@ struct CoarseSolver {
     }
     return minres() ? minres_iter(mw, C, x, n, k, tol, scr, scr_bytes) : gcr_iter(w, A, nullptr, x, n, k, tol * tol);
   }
-  // even-odd: x_o = D_oo^-1 (b_o - D_oe x_e), x = (x_e, x_o)
+  // even-odd: the pending MINRES update, then x_o = D_oo^-1 (b_o - D_oe x_e), x =
+  // (x_e, x_o)
   mglma_status finish(const Vec& b, Vec& x) {
     if (!eo()) return MGLMA_OK;
+    Vec xn = xe;
+    xn.nrhs = b.nrhs;
+    MG_CHECK(minres_end(mw, C, xn, b.nrhs, true));
     return coarse_eo_reconstruct(ctx, C, b.p, xe.p, x.p, b.nrhs, MGLMA_FP32, scr, scr_bytes, s);
   }
   // captures the init and cycle graphs of n RHS into G; on any failure G is

@@ -106,7 +106,7 @@ mglma_status coarse_eo_setup(mglma_ctx ctx, mglma_coarse_s* C, cudaStream_t s);
 // its last launch: FP32 on the tensor cores, one RHS tile
 bool coarse_schur_dot_ok(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs, int prec);
 // x_imaged (with dot_out only): the scratch's first half already holds the
-// image of X_e (coarse_x_image_half / minres_update_image)
+// image of X_e (coarse_x_image_half / lanczos_step)
 mglma_status coarse_schur_apply(mglma_ctx ctx, const mglma_coarse_s* C, const void* Xe, void* Ye, int nrhs, int prec,
                                 int mode, void* scratch, size_t scratch_bytes, cudaStream_t s,
                                 double2* dot_out = nullptr, bool x_imaged = false);
@@ -158,10 +158,16 @@ int coarse_tc_nt(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs);
 // launch would write it
 mglma_status coarse_x_image_half(mglma_ctx ctx, const mglma_coarse_s* C, const void* X, int nrhs, void* image,
                                  cudaStream_t s);
-// minres_update on FP32 half-lattice fields that also writes the image of
-// the scaled z (the next Lanczos vector) into image, as coarse_x_image_half
-mglma_status minres_update_image(mglma_ctx ctx, const mglma_coarse_s* C, const double* cf, int stride, const Vec& v,
-                                 const Vec& w1, const Vec& w2, Vec& wn, Vec& x, Vec& z, void* image, cudaStream_t s);
+// one MINRES iteration after the operator on unnormalised Lanczos vectors (FP32
+// half-lattice fields, see lanczos_step_kernel): y = Q u_k on entry, u_(k+1) on
+// return; w1 = w_(k-2), w2 = w_(k-3) on entry and w_(k-1) on return; the image of
+// u_(k+1) as coarse_x_image_half would write it.  minres_flush applies the update
+// the last iteration left pending (cf = its MR_CF coefficients) to x.
+mglma_status lanczos_step(mglma_ctx ctx, const mglma_coarse_s* C, double* st, int cap, const double2* dot, int* active,
+                          double tol, const Vec& u, const Vec& uo, Vec& y, const Vec& w1, Vec& w2, Vec& x, void* image,
+                          cudaStream_t s);
+mglma_status minres_flush(mglma_ctx ctx, const double* cf, int cap, const Vec& u, const Vec& w1, const Vec& w2, Vec& x,
+                          cudaStream_t s);
 size_t coarse_tc_half_image_bytes(const mglma_coarse_s* C, int nrhs);
 mglma_status coarse_tc_image_blocks(mglma_ctx ctx, const double2* A64, int64_t V1, int n2, int nslots,
                                     uint16_t** img, cudaStream_t s);
