@@ -4,10 +4,13 @@
 // (Fig. A).  Slot d < 4 couples y to y + mu, 4..7 to y - mu, 8 to y itself.
 //
 // Build (FP64, setup): for a batch of basis columns j', the fine field equal
-// to phi_{j'} on every block is pushed through each hop-slot piece of D (the
-// hops that leave a block through the face of slot d, or for slot 8 the
-// clover term plus every hop inside the block) and restricted with R0; column
-// j' of Dhat_d(y) is the result at block y.
+// to phi_{j'} on every block goes through the hop-slot pieces of D for d = 0..3
+// (the hops that leave a block through its +mu face) and 8 (the clover term plus
+// every hop inside the block) and is restricted with R0, over the face's sites
+// alone for d < 4; column j' of Dhat_d(y) is the result at block y.  The backward
+// slots follow from gamma5-hermiticity, Dhat_{-mu}(y + mu) = g5 Dhat_{+mu}(y)^dag
+// g5.  FP64-pipe bound: with nine slots restricted over whole blocks 32x16^3, Nv
+// 16 spent 50 ms in R0.
 //
 // Apply: Y(y) = sum_d Dhat_d(y) X(nbr_d(y)) for many right-hand sides.  The
 // adjoint uses gamma5-hermiticity on the coarse grid, Dhat^dag = g5 Dhat g5
@@ -91,11 +94,27 @@ mglma_status coarse_scale_convert(mglma_ctx ctx, const void* src, int sprec, voi
 }
 
 // ------------------------------------------------------------ build helpers
-__global__ void unit_columns_kernel(double2* __restrict__ u, int nb, int64_t V1, int n2, int j0) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)nb * V1 * n2) return;
-  const int j = (int)(i % n2), r = (int)(i / ((size_t)V1 * n2));
-  u[i] = make_double2(j == j0 + r ? 1.0 : 0.0, 0.0);
+// A[y][4 + mu] = g5 A[y - mu][mu]^dag g5; one CTA per (block, direction)
+__global__ void backward_slots_kernel(double2* __restrict__ A, LatIdx q, int n2) {
+  const int64_t y = blockIdx.x;
+  const int mu = blockIdx.y;
+  int x[4];
+  site_coords(q, y, x);
+  int64_t z = 0;
+  switch (mu) {
+    case 0: z = nbr_bwd(q, y, x, 0); break;
+    case 1: z = nbr_bwd(q, y, x, 1); break;
+    case 2: z = nbr_bwd(q, y, x, 2); break;
+    default: z = nbr_bwd(q, y, x, 3); break;
+  }
+  const double2* src = A + ((size_t)z * 9 + mu) * n2 * n2;
+  double2* dst = A + ((size_t)y * 9 + 4 + mu) * n2 * n2;
+  for (int e = threadIdx.x; e < n2 * n2; e += blockDim.x) {
+    const int j = e / n2, i = e % n2;  // column j, row i of the target
+    const double2 v = src[(size_t)i * n2 + j];
+    const double s = (i < n2 / 2) == (j < n2 / 2) ? 1.0 : -1.0;
+    dst[e] = make_double2(s * v.x, -s * v.y);
+  }
 }
 
 // A64[y][d][j0 + r][i] = C[r][y][i]
@@ -298,11 +317,9 @@ mglma_status mglma_coarse_build(mglma_ctx ctx, mglma_gauge G, mglma_subspace S, 
   mglma_status st = MGLMA_OK;
   {  // column work fields, returned to the pool at the end of this scope
     FreeList fl(ctx, s);
-    double2 *U1 = nullptr, *C = nullptr;
+    double2* C = nullptr;
     Spinor Phi, H;
-    st = dalloc(ctx, (void**)&U1, (size_t)NB * g.V1 * n2 * sizeof(double2), s);
-    fl.add(U1);
-    if (st == MGLMA_OK) st = dalloc(ctx, (void**)&C, (size_t)NB * g.V1 * n2 * sizeof(double2), s);
+    st = dalloc(ctx, (void**)&C, (size_t)NB * g.V1 * n2 * sizeof(double2), s);
     fl.add(C);
     if (st == MGLMA_OK) st = alloc_spinor(ctx, Phi, MGLMA_FP64, NB, g.V, s);
     fl.add(Phi.p);
@@ -312,20 +329,21 @@ mglma_status mglma_coarse_build(mglma_ctx ctx, mglma_gauge G, mglma_subspace S, 
       const int nb = std::min(NB, n2 - j0);
       Phi.nrhs = H.nrhs = nb;
       const size_t nu = (size_t)nb * g.V1 * n2;
-      {
-        ProfScope ps(ctx, K_SETUP, s);
-        unit_columns_kernel<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(U1, nb, g.V1, n2, j0);
-      }
-      st = prolong_coarse(ctx, S, U1, Phi, false, s);
-      for (int d = 0; st == MGLMA_OK && d < 9; ++d) {
+      st = basis_columns(ctx, S, j0, Phi, s);
+      for (int d : {0, 1, 2, 3, 8}) {
+        if (st != MGLMA_OK) break;
         st = dslash_slot64_batch(ctx, G, g.b, Phi, H, d, s);
-        if (st == MGLMA_OK) st = restrict_fine(ctx, S, H, C, s);
+        if (st == MGLMA_OK) st = restrict_face64(ctx, S, H, C, d < 4 ? d : -1, s);
         if (st == MGLMA_OK) {
           ProfScope ps(ctx, K_SETUP, s);
           scatter_columns_kernel<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(C, Cc->A64, nb, g.V1, n2, j0, d);
         }
       }
     }
+  }
+  if (st == MGLMA_OK) {
+    ProfScope ps(ctx, K_SETUP, s);
+    backward_slots_kernel<<<dim3((unsigned)g.V1, 4), 256, 0, s>>>(Cc->A64, make_latidx(g.Lb), n2);
   }
   if (st == MGLMA_OK && cudaGetLastError() != cudaSuccess) st = fail(MGLMA_ERR_CUDA, "coarse_build: launch failed");
   if (st == MGLMA_OK) st = coarse_store_copies(ctx, Cc, store, s);

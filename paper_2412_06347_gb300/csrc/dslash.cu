@@ -611,6 +611,7 @@ __global__ void __launch_bounds__(128) dslash_slot_kernel(const double2* __restr
   if (site >= V) return;
   int x[4];
   site_coords(a.q, site, x);
+  if (a.slot < 8 && !crosses(x, a.b, a.slot)) return;  // off the face: not written, not read
   Cx<double> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = cx(0.0, 0.0);

@@ -372,7 +372,7 @@ mglma_status eo_embed(mglma_ctx, const mglma_gauge_s* G, const Spinor& e, Spinor
 mglma_status eo_extract(mglma_ctx, const mglma_gauge_s* G, const Spinor& f, Spinor& e, cudaStream_t s);
 // single hop-slot pieces of D in FP64, used to assemble the coarse operator:
 // slot d < 8: the hop term of slot d at sites whose hop leaves their block
-// (zero elsewhere); slot 8: clover term plus every hop that stays in the block.
+// (other sites are not written); slot 8: clover term plus every hop that stays in the block.
 mglma_status dslash_slot64_batch(mglma_ctx, const mglma_gauge_s* G, const int block[4], const Spinor& in,
                                  Spinor& out, int slot, cudaStream_t s);
 

@@ -181,10 +181,30 @@ __device__ __forceinline__ Cx<double> fine_get<double>(const void* f, int64_t V,
 
 // ------------------------------------------------------------ R0: restrict
 // out[r][y][j] = sum_{k in B_y} sum_q conj(phi_{y j}(k)_q) psi_r(site(y,k))_{6 alpha(j) + q}
+// With slot >= 0 the sum runs over the sites of the block's face towards that hop
+// slot alone (the fine field vanishes elsewhere: set-up of the coarse operator).
 // One CTA per (block, RHS tile): the block's spinors are staged in shared
 // memory (component-major, conflict-free), each warp owns a set of dofs j,
 // lanes stride over the sites reading the basis coalesced, and a warp-shuffle
 // reduction finishes each inner product.
+// site-in-block index of the f-th site of the face hop slot d leaves through
+__device__ __forceinline__ int face_site(const BlockGeo& g, int d, int f) {
+  const int mu = d & 3;
+  int k = 0, stride = 1;
+  for (int m = 3; m >= 0; --m) {
+    int c;
+    if (m == mu) {
+      c = d < 4 ? g.b[m] - 1 : 0;
+    } else {
+      c = f % g.b[m];
+      f /= g.b[m];
+    }
+    k += c * stride;
+    stride *= g.b[m];
+  }
+  return k;
+}
+
 constexpr int RP_THREADS = 256;
 constexpr int RP_CHUNK = 128;  // sites per shared-memory chunk
 
@@ -192,7 +212,7 @@ template <typename R, typename B, int NRT, int JW>
 __global__ void __launch_bounds__(RP_THREADS) restrict_kernel(const void* __restrict__ fine, int nrhs,
                                                               const void* __restrict__ basis,
                                                               const float* __restrict__ scale, BlockGeo g, int n2,
-                                                              Cx<R>* __restrict__ out) {
+                                                              Cx<R>* __restrict__ out, int slot) {
   extern __shared__ unsigned char smraw[];
   Cx<R>* sm = reinterpret_cast<Cx<R>*>(smraw);  // [NRT][12][RP_CHUNK]
   // RHS tiles fastest: the CTAs of one block run together and share its basis in L2
@@ -209,11 +229,17 @@ __global__ void __launch_bounds__(RP_THREADS) restrict_kernel(const void* __rest
     for (int r = 0; r < NRT; ++r) acc[a][r] = cx<R>(0, 0);
 
   __shared__ int64_t site_of[RP_CHUNK];
+  __shared__ int k_of[RP_CHUNK];
   const int nv = n2 / 2;
-  for (int k0 = 0; k0 < g.nB; k0 += RP_CHUNK) {
-    const int ck = min(RP_CHUNK, g.nB - k0);
+  const int nk = slot < 0 ? g.nB : g.nB / g.b[slot & 3];
+  for (int k0 = 0; k0 < nk; k0 += RP_CHUNK) {
+    const int ck = min(RP_CHUNK, nk - k0);
     __syncthreads();
-    for (int kk = threadIdx.x; kk < ck; kk += RP_THREADS) site_of[kk] = block_site(g, y, k0 + kk);
+    for (int kk = threadIdx.x; kk < ck; kk += RP_THREADS) {
+      const int k = slot < 0 ? k0 + kk : face_site(g, slot, k0 + kk);
+      k_of[kk] = k;
+      site_of[kk] = block_site(g, y, k);
+    }
     __syncthreads();
     if constexpr (sizeof(R) == 4) {  // 16-byte loads: two complex components per load
       for (int idx = threadIdx.x; idx < NRT * 6 * ck; idx += RP_THREADS) {
@@ -247,7 +273,7 @@ __global__ void __launch_bounds__(RP_THREADS) restrict_kernel(const void* __rest
           const int j = warp + a * NW;
           if (j >= n2 || (j >= nv) != (al == 1)) continue;
           Cx<R> ph[6];
-          BIO<B>::template load<R>(basis, scale, (size_t)y * n2 + j, g.nB, k0 + kk, ph);
+          BIO<B>::template load<R>(basis, scale, (size_t)y * n2 + j, g.nB, k_of[kk], ph);
 #pragma unroll
           for (int r = 0; r < NRT; ++r)
 #pragma unroll
@@ -837,7 +863,7 @@ static int subspace_smem_restrict(int nrt, int rbytes) { return nrt * 12 * RP_CH
 
 template <typename R, typename B, int NRT, int JW>
 static mglma_status launch_restrict_jw(const mglma_subspace_s* S, const void* fine, int nrhs, const void* basis,
-                                       void* out, cudaStream_t s) {
+                                       void* out, cudaStream_t s, int slot) {
   const BlockGeo g = S->geo;
   const int smem = subspace_smem_restrict(NRT, sizeof(R));
   static bool attr_set = false;
@@ -847,7 +873,7 @@ static mglma_status launch_restrict_jw(const mglma_subspace_s* S, const void* fi
   }
   const unsigned grid = (unsigned)(g.V1 * ((nrhs + NRT - 1) / NRT));
   restrict_kernel<R, B, NRT, JW><<<grid, RP_THREADS, smem, s>>>(fine, nrhs, basis, S->scale16, g, 2 * S->nv,
-                                                                reinterpret_cast<Cx<R>*>(out));
+                                                                reinterpret_cast<Cx<R>*>(out), slot);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
@@ -855,16 +881,16 @@ static mglma_status launch_restrict_jw(const mglma_subspace_s* S, const void* fi
 // dofs per warp: ceil(2 Nv / 8) rounded up to an instantiated width
 template <typename R, typename B, int NRT>
 static mglma_status launch_restrict(const mglma_subspace_s* S, const void* fine, int nrhs, const void* basis,
-                                    void* out, cudaStream_t s) {
+                                    void* out, cudaStream_t s, int slot = -1) {
   const int jw = (2 * S->nv + 7) / 8;
-  if (jw <= 1) return launch_restrict_jw<R, B, NRT, 1>(S, fine, nrhs, basis, out, s);
-  if (jw <= 2) return launch_restrict_jw<R, B, NRT, 2>(S, fine, nrhs, basis, out, s);
-  if (jw <= 3) return launch_restrict_jw<R, B, NRT, 3>(S, fine, nrhs, basis, out, s);
-  if (jw <= 4) return launch_restrict_jw<R, B, NRT, 4>(S, fine, nrhs, basis, out, s);
-  if (jw <= 6) return launch_restrict_jw<R, B, NRT, 6>(S, fine, nrhs, basis, out, s);
-  if (jw <= 8) return launch_restrict_jw<R, B, NRT, 8>(S, fine, nrhs, basis, out, s);
-  if (jw <= 12) return launch_restrict_jw<R, B, NRT, 12>(S, fine, nrhs, basis, out, s);
-  return launch_restrict_jw<R, B, NRT, 16>(S, fine, nrhs, basis, out, s);
+  if (jw <= 1) return launch_restrict_jw<R, B, NRT, 1>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 2) return launch_restrict_jw<R, B, NRT, 2>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 3) return launch_restrict_jw<R, B, NRT, 3>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 4) return launch_restrict_jw<R, B, NRT, 4>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 6) return launch_restrict_jw<R, B, NRT, 6>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 8) return launch_restrict_jw<R, B, NRT, 8>(S, fine, nrhs, basis, out, s, slot);
+  if (jw <= 12) return launch_restrict_jw<R, B, NRT, 12>(S, fine, nrhs, basis, out, s, slot);
+  return launch_restrict_jw<R, B, NRT, 16>(S, fine, nrhs, basis, out, s, slot);
 }
 
 template <typename R, typename B, int NRT>
@@ -1014,6 +1040,47 @@ mglma_status restrict_fine(mglma_ctx ctx, const mglma_subspace_s* S, const Spino
   }
   if (S->phi16) return launch_restrict<float, __half, 4>(S, in.p, in.nrhs, S->phi16, out_coarse, s);
   return launch_restrict<float, float, 4>(S, in.p, in.nrhs, S->phi32, out_coarse, s);
+}
+
+// FP64 fine fields r = 0..nb-1 equal to basis column j0 + r on every block
+template <typename B>
+__global__ void basis_columns_kernel(const void* __restrict__ basis, const float* __restrict__ scale, BlockGeo g,
+                                     int nv, int j0, double2* __restrict__ out) {
+  const int k = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) % g.nB);
+  const int64_t y = (int64_t)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) / g.nB);
+  if (y >= g.V1) return;
+  const int r = blockIdx.y, j = j0 + r, chi = j >= nv ? 1 : 0;
+  Cx<double> v[6];
+  BIO<B>::template load<double>(basis, scale, (size_t)y * 2 * nv + j, g.nB, k, v);
+  double2* p = out + (size_t)r * 12 * g.V + block_site(g, y, k);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    p[(size_t)(6 * chi + q) * g.V] = make_double2(v[q].re, v[q].im);
+    p[(size_t)(6 * (1 - chi) + q) * g.V] = make_double2(0, 0);
+  }
+}
+
+mglma_status basis_columns(mglma_ctx ctx, const mglma_subspace_s* S, int j0, Spinor& out, cudaStream_t s) {
+  ProfScope ps(ctx, K_SETUP, s);
+  const dim3 g((unsigned)((S->geo.V + 255) / 256), (unsigned)out.nrhs, 1);
+  if (S->phi64)
+    basis_columns_kernel<double><<<g, 256, 0, s>>>(S->phi64, nullptr, S->geo, S->nv, j0, (double2*)out.p);
+  else if (S->phi16)
+    basis_columns_kernel<__half><<<g, 256, 0, s>>>(S->phi16, S->scale16, S->geo, S->nv, j0, (double2*)out.p);
+  else
+    basis_columns_kernel<float><<<g, 256, 0, s>>>(S->phi32, nullptr, S->geo, S->nv, j0, (double2*)out.p);
+  MG_LAUNCH_CHECK();
+  return MGLMA_OK;
+}
+
+mglma_status restrict_face64(mglma_ctx ctx, const mglma_subspace_s* S, const Spinor& in, void* out_coarse, int slot,
+                             cudaStream_t s) {
+  ProfScope ps(ctx, K_RESTRICT, s, transfer_bytes(S, in.prec, in.nrhs) / (slot < 0 ? 1 : S->geo.b[slot & 3]),
+               8.0 * S->geo.V * 12.0 * S->nv * in.nrhs / (slot < 0 ? 1 : S->geo.b[slot & 3]));
+  if (in.prec != MGLMA_FP64 || slot > 7) return fail(MGLMA_ERR_INVALID, "restrict_face64: FP64 fields, slots 0..7");
+  if (S->phi64) return launch_restrict<double, double, 2>(S, in.p, in.nrhs, S->phi64, out_coarse, s, slot);
+  if (S->phi16) return launch_restrict<double, __half, 2>(S, in.p, in.nrhs, S->phi16, out_coarse, s, slot);
+  return launch_restrict<double, float, 2>(S, in.p, in.nrhs, S->phi32, out_coarse, s, slot);
 }
 
 mglma_status prolong_coarse(mglma_ctx ctx, const mglma_subspace_s* S, const void* in_coarse, Spinor& out,

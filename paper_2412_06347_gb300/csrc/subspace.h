@@ -64,6 +64,12 @@ namespace mglma {
 
 mglma_status restrict_fine(mglma_ctx ctx, const mglma_subspace_s* S, const Spinor& in, void* out_coarse,
                            cudaStream_t s);
+// set-up of the coarse operator (FP64; a lean subspace's stored copy is widened):
+// fine fields equal to the basis columns j0 .. j0 + out.nrhs - 1 on every block,
+// and R0 over the sites of each block's face of hop slot 0..7 alone (-1: all)
+mglma_status basis_columns(mglma_ctx ctx, const mglma_subspace_s* S, int j0, Spinor& out, cudaStream_t s);
+mglma_status restrict_face64(mglma_ctx ctx, const mglma_subspace_s* S, const Spinor& in, void* out_coarse, int slot,
+                             cudaStream_t s);
 mglma_status prolong_coarse(mglma_ctx ctx, const mglma_subspace_s* S, const void* in_coarse, Spinor& out,
                             bool accumulate, cudaStream_t s);
 // n_smooth MR steps on D v = 0 in the precision of v
