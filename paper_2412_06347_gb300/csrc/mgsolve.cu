@@ -850,6 +850,7 @@ struct TwoLevel {
   bool fused = false;      // fused MR steps on BF16 s, t
   bool tc_r0 = false;      // R0 on the tensor cores (BF16 operands; the coarse solve is BF16 already)
   bool tc_t0 = false;      // T0 on the tensor cores (BF16 operands)
+  bool half_r0 = false, half_t0 = false;  // ... on half fields
   bool capturing = false;  // recording into a graph: the coarse loop runs on the device
   // even-odd form: r and z are FP32 half fields (even sites) of the Schur
   // system, the odd part of the full residual being zero
@@ -878,8 +879,12 @@ struct TwoLevel {
     // solve takes the rounded preconditioner; measured: same FGCR and coarse
     // iteration counts as FP32 at 64x32^3), FP32 otherwise
     fused = eo || (p->nu > 1 && dslash_mr_fused(ctx, G, n));
-    tc_r0 = n >= 8 && restrict_tc_supported(C->sub);
-    tc_t0 = n >= 8 && prolong_tc_supported(C->sub);
+    // in even-odd form on the even sites where the half blocks fit, else on a
+    // full field
+    half_r0 = eo && n >= 8 && restrict_tc_supported(C->sub, true);
+    half_t0 = eo && n >= 8 && prolong_tc_supported(C->sub, true);
+    tc_r0 = n >= 8 && (half_r0 || restrict_tc_supported(C->sub));
+    tc_t0 = n >= 8 && (half_t0 || prolong_tc_supported(C->sub));
     sv = r;
     sv.nrhs = n;
     sv.p = nullptr;
@@ -894,7 +899,7 @@ struct TwoLevel {
       wo.p = full.p = nullptr;
       full.n = 2 * r.n;
       MG_CHECK(dalloc(ctx, &wo.p, wo.bytes(), s));
-      MG_CHECK(dalloc(ctx, &full.p, full.bytes(), s));
+      if (!half_r0 || !half_t0) MG_CHECK(dalloc(ctx, &full.p, full.bytes(), s));
     }
     const int64_t V = C->sub->geo.V;
     MG_CHECK(dalloc(ctx, (void**)&part,
@@ -926,7 +931,11 @@ struct TwoLevel {
       Vec f = full;
       f.nrhs = n;
       rs = zs = as_spinor(f, V);
-      MG_CHECK(eo_embed(ctx, G, rh, rs, s));
+      if (half_r0)
+        rs = rh;
+      else
+        MG_CHECK(eo_embed(ctx, G, rh, rs, s));
+      if (half_t0) zs = zh;
     }
     if (tc_r0)
       MG_CHECK(restrict_tc(ctx, const_cast<mglma_subspace_s*>(S), rs, b1n.p, s));
@@ -941,7 +950,7 @@ struct TwoLevel {
     else
       MG_CHECK(prolong_coarse(ctx, S, e1n.p, zs, false, s));
     if (eo) {
-      MG_CHECK(eo_extract(ctx, G, zs, zh, s));
+      if (!half_t0) MG_CHECK(eo_extract(ctx, G, zs, zh, s));
       return smooth_eo(rh, zh, n);
     }
     if (p->nu > 0) {

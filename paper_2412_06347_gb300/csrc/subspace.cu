@@ -1429,6 +1429,8 @@ void mglma_subspace_free(mglma_subspace S) {
   cudaFree(S->scale16);
   cudaFree(S->rt_img);
   cudaFree(S->pt_img);
+  cudaFree(S->rt_img_eo);
+  cudaFree(S->pt_img_eo);
   cudaFree(S->rt_err);
   delete S;
 }

@@ -27,6 +27,7 @@ struct mglma_subspace_s {
   bool lean = false;         // built without an FP64 copy (phi64 stays NULL)
   uint16_t* rt_img = nullptr;  // cache: BF16 image of the basis for the tensor-core R0 (transfer_tc.cu), built on first use
   uint16_t* pt_img = nullptr;  // cache: BF16 image of the basis for the tensor-core T0, built on first use
+  uint16_t *rt_img_eo = nullptr, *pt_img_eo = nullptr;  // the same for the even sites alone (the even-odd solve)
   int* rt_err = nullptr;       // the error flag of both tensor-core transfer kernels
 };
 
@@ -130,13 +131,16 @@ mglma_status coarse_schur_full(mglma_ctx ctx, mglma_coarse_s* C, const void* X, 
 // [rhs][V1][2Nv] out, BF16 operands (basis imaged on first use); needs
 // Nv % 8 == 0, Nv <= 32, 64 | |B| <= 512.  restrict_tc_check reports a
 // bounded wait that gave up.
-bool restrict_tc_supported(const mglma_subspace_s* S);
+// A half field (in.V = V / 2) holds the even sites and stands for a field that
+// vanishes on the odd ones; supported asks with |B| / 2 for |B| then.
+bool restrict_tc_supported(const mglma_subspace_s* S, bool half = false);
 mglma_status restrict_tc(mglma_ctx ctx, mglma_subspace_s* S, const Spinor& in, void* out, cudaStream_t s);
 mglma_status restrict_tc_check(const mglma_subspace_s* S, cudaStream_t s);
 // T0 on the tensor cores: FP32 coarse [rhs][V1][2Nv] in, FP32 fine fields
 // out (overwritten), BF16 operands; needs Nv % 8 == 0, Nv <= 32,
 // 128 | |B| <= 512.  Its timeouts are reported by restrict_tc_check too.
-bool prolong_tc_supported(const mglma_subspace_s* S);
+// A half field (out.V = V / 2) receives the even sites.
+bool prolong_tc_supported(const mglma_subspace_s* S, bool half = false);
 mglma_status prolong_tc(mglma_ctx ctx, mglma_subspace_s* S, const void* in_coarse, Spinor& out, cudaStream_t s);
 // scratch the FP32 (tensor-core) even-odd calls need for nrhs RHS
 size_t coarse_eo_scratch_bytes(const mglma_coarse_s* C, int nrhs);

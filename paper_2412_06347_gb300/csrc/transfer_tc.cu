@@ -71,12 +71,54 @@ __device__ __forceinline__ int64_t rt_block_site(const BlockGeo& g, int64_t y, i
   return s;
 }
 
+// Even sites only (the even-odd solve: the residual vanishes on the odd sites and
+// the correction is used on the even ones): a geometry with half set holds nB =
+// |B| / 2 and V / 2, and site k of block y is its k-th even site -- the sites are
+// paired along `pair`, the last direction of even side, and each pair has one.
+struct TcGeo {
+  BlockGeo g;
+  int half = 0, pair = 3, nBfull = 0;
+};
+static TcGeo tc_geo(const BlockGeo& g, bool half) {
+  TcGeo t;
+  t.g = g;
+  t.nBfull = g.nB;
+  if (half) {
+    t.half = 1;
+    t.g.nB /= 2;
+    t.g.V /= 2;
+    while (t.pair > 0 && g.b[t.pair] % 2) --t.pair;
+  }
+  return t;
+}
+// site-in-block index and field index of site k
+__device__ __forceinline__ int rt_k(const TcGeo& t, int64_t y, int k) {
+  if (!t.half) return k;
+  int kc[4], par = 0, u = k;
+  int64_t q = y;
+  for (int m = 3; m >= 0; --m) {
+    const int side = m == t.pair ? t.g.b[m] / 2 : t.g.b[m];
+    kc[m] = u % side;
+    u /= side;
+    if (m != t.pair) par += kc[m] + (int)(q % t.g.Lb[m]) * t.g.b[m];
+    q /= t.g.Lb[m];
+  }
+  int r = 0;
+  for (int m = 0; m < 4; ++m) r = r * t.g.b[m] + (m == t.pair ? 2 * kc[m] + (par & 1) : kc[m]);
+  return r;
+}
+__device__ __forceinline__ int64_t rt_site(const TcGeo& t, int64_t y, int k) {
+  const int64_t s = rt_block_site(t.g, y, rt_k(t, y, k));
+  return t.half ? s >> 1 : s;
+}
+
 // the basis image, one thread per BF16 value: [y][alpha][seg][kc][g][ri][e]
 // with seg = c (nB / 64) + og, kc = (o 2 + h) 2 + p, j = alpha Nv + 8 g + ri,
 // site k = 64 og + 8 o + e, component q = 2c + h
 template <typename B>
-__global__ void rt_image_kernel(const void* __restrict__ basis, const float* __restrict__ scale, BlockGeo g, int nv,
+__global__ void rt_image_kernel(const void* __restrict__ basis, const float* __restrict__ scale, TcGeo tg, int nv,
                                 uint16_t* __restrict__ img) {
+  const BlockGeo& g = tg.g;
   const int GA = nv / 8, nog = g.nB / RT_SEG, nseg = 3 * nog;
   const size_t per_seg = (size_t)RT_CH * GA * 64;
   const size_t per_y = 2 * (size_t)nseg * per_seg;
@@ -93,17 +135,17 @@ __global__ void rt_image_kernel(const void* __restrict__ basis, const float* __r
   const int c = seg / nog, og = seg % nog;
   const int n2 = 2 * nv;
   const int j = alpha * nv + 8 * gg + ri;
-  const int k = RT_SEG * og + 8 * o + e;
+  const int k = rt_k(tg, y, RT_SEG * og + 8 * o + e);
   const size_t yj = (size_t)y * n2 + j;
   float re, im;
   if (sizeof(B) == 2) {
-    uint2 v = __ldg(reinterpret_cast<const uint2*>(basis) + (yj * 3 + c) * g.nB + k);
+    uint2 v = __ldg(reinterpret_cast<const uint2*>(basis) + (yj * 3 + c) * tg.nBfull + k);
     const float2 f = __half22float2(*reinterpret_cast<__half2*>(h ? &v.y : &v.x));
     const float sc = __ldg(scale + yj);
     re = f.x * sc;
     im = f.y * sc;
   } else {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(basis) + (yj * 3 + c) * g.nB + k);
+    const float4 v = __ldg(reinterpret_cast<const float4*>(basis) + (yj * 3 + c) * tg.nBfull + k);
     re = h ? v.z : v.x;
     im = h ? v.w : v.y;
   }
@@ -137,7 +179,8 @@ struct RtRun {
   int* err;
 };
 
-__global__ void __launch_bounds__(RT_THREADS, 2) restrict_tc_kernel(RtRun run, BlockGeo g, int nv, int nstages) {
+__global__ void __launch_bounds__(RT_THREADS, 2) restrict_tc_kernel(RtRun run, TcGeo tg, int nv, int nstages) {
+  const BlockGeo& g = tg.g;
   extern __shared__ __align__(1024) uint8_t sm[];
   const int GA = nv / 8, nog = g.nB / RT_SEG, nseg = 3 * nog, n2 = 2 * nv;
   const uint32_t a_bytes = (uint32_t)RT_CH * GA * 128;
@@ -198,7 +241,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2) restrict_tc_kernel(RtRun run, B
       // all producers stop together (a wait gave up); the same barrier
       // guarantees the previous unit's site table is consumed
       if (rt_producers_any(!ok || *abrt)) break;
-      for (int k = tid; k < g.nB; k += 128) site_of[k] = rt_block_site(g, y, k);
+      for (int k = tid; k < g.nB; k += 128) site_of[k] = rt_site(tg, y, k);
       asm volatile("bar.sync 1, 128;" ::: "memory");
       const int rr = t * RT_NT + r;
       for (int alpha = 0; alpha < 2 && ok; ++alpha) {
@@ -375,8 +418,9 @@ constexpr int PT_PAIRS = 2;      // accumulator pairs (tiles h = 0, 1 of one flo
 // the T0 basis image, one thread per BF16 value: [y][alpha][m][kc][g][ri][e],
 // row 8 g + ri = site k - 128 half of the tile, K = 8 kc + e = p Nv + jj
 template <typename B>
-__global__ void pt_image_kernel(const void* __restrict__ basis, const float* __restrict__ scale, BlockGeo g, int nv,
+__global__ void pt_image_kernel(const void* __restrict__ basis, const float* __restrict__ scale, TcGeo tg, int nv,
                                 uint16_t* __restrict__ img) {
+  const BlockGeo& g = tg.g;
   const int KC = nv / 4, nhalf = g.nB / 128, ntile = 6 * nhalf;
   const size_t per_tile = (size_t)KC * 16 * 64;
   const size_t per_y = 2 * (size_t)ntile * per_tile;
@@ -393,17 +437,17 @@ __global__ void pt_image_kernel(const void* __restrict__ basis, const float* __r
   const int K = 8 * kc + e, p = K / nv, jj = K % nv;
   const int n2 = 2 * nv;
   const int j = alpha * nv + jj;
-  const int k = 128 * half + 8 * gg + ri;
+  const int k = rt_k(tg, y, 128 * half + 8 * gg + ri);
   const size_t yj = (size_t)y * n2 + j;
   float re, im;
   if (sizeof(B) == 2) {
-    uint2 v = __ldg(reinterpret_cast<const uint2*>(basis) + (yj * 3 + cq) * g.nB + k);
+    uint2 v = __ldg(reinterpret_cast<const uint2*>(basis) + (yj * 3 + cq) * tg.nBfull + k);
     const float2 f = __half22float2(*reinterpret_cast<__half2*>(h ? &v.y : &v.x));
     const float sc = __ldg(scale + yj);
     re = f.x * sc;
     im = f.y * sc;
   } else {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(basis) + (yj * 3 + cq) * g.nB + k);
+    const float4 v = __ldg(reinterpret_cast<const float4*>(basis) + (yj * 3 + cq) * tg.nBfull + k);
     re = h ? v.z : v.x;
     im = h ? v.w : v.y;
   }
@@ -424,7 +468,8 @@ struct PtRun {
 // writes each unit's coefficient image into one of two buffers.  The two
 // tiles h = 0, 1 of one component pair go to the two halves of an
 // accumulator pair, so each site's float4 chunk is stored whole.
-__global__ void __launch_bounds__(PT_THREADS, 2) prolong_tc_kernel(PtRun run, BlockGeo g, int nv, int nstages) {
+__global__ void __launch_bounds__(PT_THREADS, 2) prolong_tc_kernel(PtRun run, TcGeo tg, int nv, int nstages) {
+  const BlockGeo& g = tg.g;
   extern __shared__ __align__(1024) uint8_t sm[];
   const int KC = nv / 4, nhalf = g.nB / 128, ntile = 6 * nhalf, n2 = 2 * nv;
   const uint32_t a_bytes = (uint32_t)KC * 16 * 128;
@@ -618,7 +663,7 @@ __global__ void __launch_bounds__(PT_THREADS, 2) prolong_tc_kernel(PtRun run, Bl
       const int64_t y = u / ntiles;
       const int t = (int)(u % ntiles);
       int64_t site_h[4];
-      for (int hf = 0; hf < nhalf; ++hf) site_h[hf] = rt_block_site(g, y, 128 * hf + kk);
+      for (int hf = 0; hf < nhalf; ++hf) site_h[hf] = rt_site(tg, y, 128 * hf + kk);
       for (int alpha = 0; alpha < 2 && ok; ++alpha)
         for (int mp = 0; mp < ntile / 2; ++mp, ++tp) {
           const uint32_t sp = tp % PT_PAIRS, aph = (tp / PT_PAIRS) & 1u;
@@ -651,34 +696,42 @@ __global__ void __launch_bounds__(PT_THREADS, 2) prolong_tc_kernel(PtRun run, Bl
 }
 
 // ============================================================ host side
-bool restrict_tc_supported(const mglma_subspace_s* S) {
-  return S->nv % 8 == 0 && S->nv <= 32 && S->geo.nB % RT_SEG == 0 && S->geo.nB <= RT_MAX_NB &&
-         (S->phi16 || S->phi32);
+bool restrict_tc_supported(const mglma_subspace_s* S, bool half) {
+  if (half && S->geo.nB % 2) return false;
+  const int nB = half ? S->geo.nB / 2 : S->geo.nB;
+  return S->nv % 8 == 0 && S->nv <= 32 && nB % RT_SEG == 0 && nB <= RT_MAX_NB && (S->phi16 || S->phi32);
 }
 
-static mglma_status rt_image_ready(mglma_ctx ctx, mglma_subspace_s* S, cudaStream_t s) {
-  if (S->rt_img) return MGLMA_OK;
-  const BlockGeo& g = S->geo;
+static mglma_status rt_image_ready(mglma_ctx ctx, mglma_subspace_s* S, const TcGeo& tg, cudaStream_t s) {
+  uint16_t*& img = tg.half ? S->rt_img_eo : S->rt_img;
+  if (img) return MGLMA_OK;
+  const BlockGeo& g = tg.g;
   const size_t n = (size_t)g.V1 * 2 * 3 * (g.nB / RT_SEG) * RT_CH * (S->nv / 8) * 64;  // BF16 values
-  MG_CUDA(cudaMalloc(&S->rt_img, n * sizeof(uint16_t)));
-  MG_CUDA(cudaMalloc(&S->rt_err, sizeof(int)));
-  MG_CUDA(cudaMemsetAsync(S->rt_err, 0, sizeof(int), s));
+  MG_CUDA(cudaMalloc(&img, n * sizeof(uint16_t)));
+  if (!S->rt_err) {
+    MG_CUDA(cudaMalloc(&S->rt_err, sizeof(int)));
+    MG_CUDA(cudaMemsetAsync(S->rt_err, 0, sizeof(int), s));
+  }
   ProfScope ps(ctx, K_SETUP, s);
   const unsigned blocks = (unsigned)((n + 255) / 256);
   if (S->phi16)
-    rt_image_kernel<__half><<<blocks, 256, 0, s>>>(S->phi16, S->scale16, g, S->nv, S->rt_img);
+    rt_image_kernel<__half><<<blocks, 256, 0, s>>>(S->phi16, S->scale16, tg, S->nv, img);
   else
-    rt_image_kernel<float><<<blocks, 256, 0, s>>>(S->phi32, nullptr, g, S->nv, S->rt_img);
+    rt_image_kernel<float><<<blocks, 256, 0, s>>>(S->phi32, nullptr, tg, S->nv, img);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
 
 mglma_status restrict_tc(mglma_ctx ctx, mglma_subspace_s* S, const Spinor& in, void* out, cudaStream_t s) {
-  if (!restrict_tc_supported(S)) return fail(MGLMA_ERR_INVALID, "restrict_tc: Nv % 8, block size or basis not supported");
-  if (in.prec != MGLMA_FP32 || in.V != S->geo.V) return fail(MGLMA_ERR_INVALID, "restrict_tc: FP32 fine fields needed");
+  const bool half = in.V == S->geo.V / 2;
+  if (!restrict_tc_supported(S, half))
+    return fail(MGLMA_ERR_INVALID, "restrict_tc: Nv % 8, block size or basis not supported");
+  if (in.prec != MGLMA_FP32 || (!half && in.V != S->geo.V))
+    return fail(MGLMA_ERR_INVALID, "restrict_tc: FP32 fine fields needed");
   if (in.nrhs == 0) return MGLMA_OK;
-  MG_CHECK(rt_image_ready(ctx, S, s));
-  const BlockGeo& g = S->geo;
+  const TcGeo tg = tc_geo(S->geo, half);
+  MG_CHECK(rt_image_ready(ctx, S, tg, s));
+  const BlockGeo& g = tg.g;
   const uint32_t stage = (uint32_t)RT_CH * (S->nv / 8) * 128 + RT_B_BYTES;
   // two CTAs per SM: half of 227 KB each, less the barriers, the site table
   // and 1 KB of static shared memory
@@ -698,7 +751,7 @@ mglma_status restrict_tc(mglma_ctx ctx, mglma_subspace_s* S, const Spinor& in, v
   const unsigned grid = (unsigned)std::min<int64_t>(units, 2 * (int64_t)ctx->sm_count);
   RtRun run;
   run.fine = (const float4*)in.p;
-  run.img = (const uint8_t*)S->rt_img;
+  run.img = (const uint8_t*)(half ? S->rt_img_eo : S->rt_img);
   run.out = (float2*)out;
   run.nrhs = in.nrhs;
   run.err = S->rt_err;
@@ -707,21 +760,24 @@ mglma_status restrict_tc(mglma_ctx ctx, mglma_subspace_s* S, const Spinor& in, v
     const double V = (double)g.V, V1 = (double)g.V1, n2 = 2.0 * S->nv, N = in.nrhs;
     ProfScope ps(ctx, K_RESTRICT, s, V * n2 * 6.0 * 4.0 * std::ceil(N / RT_NT) + N * (V * 96.0 + V1 * n2 * 8.0),
                  8.0 * V * 12.0 * S->nv * N);
-    restrict_tc_kernel<<<grid, RT_THREADS, smem, s>>>(run, g, S->nv, S_);
+    restrict_tc_kernel<<<grid, RT_THREADS, smem, s>>>(run, tg, S->nv, S_);
   }
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
 
-bool prolong_tc_supported(const mglma_subspace_s* S) {
-  return S->nv % 8 == 0 && S->nv <= 32 && S->geo.nB % 128 == 0 && S->geo.nB <= 512 && (S->phi16 || S->phi32);
+bool prolong_tc_supported(const mglma_subspace_s* S, bool half) {
+  if (half && S->geo.nB % 2) return false;
+  const int nB = half ? S->geo.nB / 2 : S->geo.nB;
+  return S->nv % 8 == 0 && S->nv <= 32 && nB % 128 == 0 && nB <= 512 && (S->phi16 || S->phi32);
 }
 
-static mglma_status pt_image_ready(mglma_ctx ctx, mglma_subspace_s* S, cudaStream_t s) {
-  if (S->pt_img) return MGLMA_OK;
-  const BlockGeo& g = S->geo;
+static mglma_status pt_image_ready(mglma_ctx ctx, mglma_subspace_s* S, const TcGeo& tg, cudaStream_t s) {
+  uint16_t*& img = tg.half ? S->pt_img_eo : S->pt_img;
+  if (img) return MGLMA_OK;
+  const BlockGeo& g = tg.g;
   const size_t n = (size_t)g.V1 * 2 * 6 * (g.nB / 128) * (S->nv / 4) * 16 * 64;  // BF16 values
-  MG_CUDA(cudaMalloc(&S->pt_img, n * sizeof(uint16_t)));
+  MG_CUDA(cudaMalloc(&img, n * sizeof(uint16_t)));
   if (!S->rt_err) {
     MG_CUDA(cudaMalloc(&S->rt_err, sizeof(int)));
     MG_CUDA(cudaMemsetAsync(S->rt_err, 0, sizeof(int), s));
@@ -729,19 +785,23 @@ static mglma_status pt_image_ready(mglma_ctx ctx, mglma_subspace_s* S, cudaStrea
   ProfScope ps(ctx, K_SETUP, s);
   const unsigned blocks = (unsigned)((n + 255) / 256);
   if (S->phi16)
-    pt_image_kernel<__half><<<blocks, 256, 0, s>>>(S->phi16, S->scale16, g, S->nv, S->pt_img);
+    pt_image_kernel<__half><<<blocks, 256, 0, s>>>(S->phi16, S->scale16, tg, S->nv, img);
   else
-    pt_image_kernel<float><<<blocks, 256, 0, s>>>(S->phi32, nullptr, g, S->nv, S->pt_img);
+    pt_image_kernel<float><<<blocks, 256, 0, s>>>(S->phi32, nullptr, tg, S->nv, img);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
 
 mglma_status prolong_tc(mglma_ctx ctx, mglma_subspace_s* S, const void* in_coarse, Spinor& out, cudaStream_t s) {
-  if (!prolong_tc_supported(S)) return fail(MGLMA_ERR_INVALID, "prolong_tc: Nv % 8, block size or basis not supported");
-  if (out.prec != MGLMA_FP32 || out.V != S->geo.V) return fail(MGLMA_ERR_INVALID, "prolong_tc: FP32 fine fields needed");
+  const bool half = out.V == S->geo.V / 2;
+  if (!prolong_tc_supported(S, half))
+    return fail(MGLMA_ERR_INVALID, "prolong_tc: Nv % 8, block size or basis not supported");
+  if (out.prec != MGLMA_FP32 || (!half && out.V != S->geo.V))
+    return fail(MGLMA_ERR_INVALID, "prolong_tc: FP32 fine fields needed");
   if (out.nrhs == 0) return MGLMA_OK;
-  MG_CHECK(pt_image_ready(ctx, S, s));
-  const BlockGeo& g = S->geo;
+  const TcGeo tg = tc_geo(S->geo, half);
+  MG_CHECK(pt_image_ready(ctx, S, tg, s));
+  const BlockGeo& g = tg.g;
   const int KC = S->nv / 4;
   const size_t a_bytes = (size_t)KC * 16 * 128, b_bytes = (size_t)KC * (RT_N / 8) * 128;
   // two CTAs per SM as for R0
@@ -761,7 +821,7 @@ mglma_status prolong_tc(mglma_ctx ctx, mglma_subspace_s* S, const void* in_coars
   const unsigned grid = (unsigned)std::min<int64_t>(units, 2 * (int64_t)ctx->sm_count);
   PtRun run;
   run.coarse = (const float2*)in_coarse;
-  run.img = (const uint8_t*)S->pt_img;
+  run.img = (const uint8_t*)(half ? S->pt_img_eo : S->pt_img);
   run.fine = (float4*)out.p;
   run.nrhs = out.nrhs;
   run.err = S->rt_err;
@@ -769,7 +829,7 @@ mglma_status prolong_tc(mglma_ctx ctx, mglma_subspace_s* S, const void* in_coars
     const double V = (double)g.V, V1 = (double)g.V1, n2 = 2.0 * S->nv, N = out.nrhs;
     ProfScope ps(ctx, K_PROLONG, s, V * n2 * 6.0 * 4.0 * std::ceil(N / RT_NT) + N * (V * 96.0 + V1 * n2 * 8.0),
                  8.0 * V * 12.0 * S->nv * N);
-    prolong_tc_kernel<<<grid, PT_THREADS, smem, s>>>(run, g, S->nv, S_);
+    prolong_tc_kernel<<<grid, PT_THREADS, smem, s>>>(run, tg, S->nv, S_);
   }
   MG_LAUNCH_CHECK();
   return MGLMA_OK;

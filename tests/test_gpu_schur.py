@@ -28,9 +28,9 @@ def ctx(m):
     c.close()
 
 
-def solve(m, ctx, L, block, nrhs, nu, t_bc, tol):
+def solve(m, ctx, L, block, nrhs, nu, t_bc, tol, nv=4):
     g = m.mglma_gauge_load(ctx, L, synthetic.gauge_links(L, 0.25, 71), 0.12, 1.2, t_bc=t_bc)
-    sub = m.mglma_subspace_build(ctx, g, block, 4, 5, 72, m.MGLMA_FP32)
+    sub = m.mglma_subspace_build(ctx, g, block, nv, 5, 72, m.MGLMA_FP32)
     C = m.mglma_coarse_build(ctx, g, sub, m.MGLMA_BF16)
     b = synthetic.random_spinors(L, nrhs, 73)
     x = np.zeros_like(b)
@@ -71,3 +71,21 @@ def test_large_half_volume(m, ctx):
     st, res = solve(m, ctx, (36, 16, 32, 32), (4, 4, 4, 4), 2, 7, -1, TOL)
     assert all(s["outer"] == 1 for s in st), st
     assert res.max() <= TOL, res
+
+
+# 8 or more RHS take R0 / T0 of the even sites on the tensor cores where half a
+# block fits them (64 / 128 sites), fewer RHS go through full fields: the same
+# preconditioner to BF16 rounding of the transfers
+@pytest.mark.parametrize("L,block", [
+    ((8, 8, 8, 8), (4, 4, 4, 4)),     # 128 even sites per block
+    ((4, 8, 8, 8), (2, 4, 4, 4)),     # 64: R0 on half fields, T0 on full ones
+    ((8, 4, 16, 8), (4, 4, 8, 4)),    # 256
+    ((6, 8, 8, 16), (3, 4, 4, 8)),    # odd side: block parities alternate; 192
+    ((8, 8, 16, 6), (4, 4, 8, 3)),    # pairs along direction 2
+    ((8, 16, 6, 6), (4, 8, 3, 3)),    # pairs along direction 1; 144 is no multiple of 64
+])
+def test_transfers_of_the_even_sites(m, ctx, L, block):
+    many, res = solve(m, ctx, L, block, 9, 7, -1, TOL, nv=8)
+    few, _ = solve(m, ctx, L, block, 2, 7, -1, TOL, nv=8)
+    assert all(s["outer"] == 1 for s in many) and res.max() <= TOL
+    assert max(abs(a["iterations"] - b["iterations"]) for a, b in zip(many, few)) <= 1, (many[:2], few)
