@@ -465,8 +465,8 @@ __global__ void __launch_bounds__(GS_THREADS) cholqr2_kernel(double2* __restrict
         double2 s = G[i * nv + j];
         for (int rr = 0; rr < tr; ++rr) {
           const double2 a = T[rr * nv + i], b = T[rr * nv + j];
-          s.x += a.x * b.x + a.y * b.y;
-          s.y += a.x * b.y - a.y * b.x;
+          s.x = fma(a.x, b.x, fma(a.y, b.y, s.x));
+          s.y = fma(a.x, b.y, fma(-a.y, b.x, s.y));
         }
         G[i * nv + j] = s;
       }
@@ -524,8 +524,8 @@ __global__ void __launch_bounds__(GS_THREADS) cholqr2_kernel(double2* __restrict
         double2 s = make_double2(0, 0);
         for (int i = 0; i <= j; ++i) {
           const double2 a = T[rr * nv + i], b = Ri[i * nv + j];
-          s.x += a.x * b.x - a.y * b.y;
-          s.y += a.x * b.y + a.y * b.x;
+          s.x = fma(a.x, b.x, fma(-a.y, b.y, s.x));
+          s.y = fma(a.x, b.y, fma(a.y, b.x, s.y));
         }
         U[j * cstride + r0 + rr] = s;
       }
