@@ -31,6 +31,7 @@
 #include <mutex>
 #include <string>
 
+#include "convert.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 #include "minres.cuh"
@@ -69,7 +70,21 @@ __device__ __forceinline__ void x_image_store(uint4* dst, int jo, int G, int NT,
   dst[(size_t)(G + jo) * N + NT + ri] = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
 }
 
-__global__ void x_image_kernel(const float2* __restrict__ X, uint4* __restrict__ XB, int64_t V1, int n2, int nrhs,
+// two consecutive dofs as the FP32 field holds them
+__device__ __forceinline__ float4 x_pair(const float2* X, size_t e) {
+  return __ldg(reinterpret_cast<const float4*>(X + e));
+}
+__device__ __forceinline__ float4 x_pair(const double2* X, size_t e) {
+  const double2 a = __ldg(X + e), b = __ldg(X + e + 1);
+  bool other = false;
+  float4 v = make_float4(d2f_fast(a.x, other), d2f_fast(a.y, other), d2f_fast(b.x, other), d2f_fast(b.y, other));
+  if (other) v = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+  return v;
+}
+
+// X: FP32 fields, or canonical complex128 ones rounded to FP32 here
+template <typename E>
+__global__ void x_image_kernel(const E* __restrict__ X, uint4* __restrict__ XB, int64_t V1, int n2, int nrhs,
                                int NT, int mode) {
   // one thread per (tile t, site z, group jo of 8 dofs, RHS r of the tile):
   // reads the group's 64 bytes of X once and writes its four 16-byte rows
@@ -85,10 +100,10 @@ __global__ void x_image_kernel(const float2* __restrict__ X, uint4* __restrict__
   const int rr = t * NT + ri;
   float re[8] = {}, im[8] = {};
   if (rr < nrhs) {
-    const float4* src = reinterpret_cast<const float4*>(X + ((size_t)rr * V1 + z) * n2 + jo * 8);
+    const size_t src = ((size_t)rr * V1 + z) * n2 + jo * 8;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      const float4 q = __ldg(src + h);
+      const float4 q = x_pair(X, src + 2 * h);
       re[2 * h] = q.x;
       im[2 * h] = q.y;
       re[2 * h + 1] = q.z;
@@ -287,6 +302,7 @@ struct TcRun {
   const uint8_t* XB;
   const uint8_t* XBself;
   float2* Y;
+  double2* Yc;  // when set, Y as canonical complex128 goes here instead
   int d_lo, d_hi;
   int par;
   float sign;
@@ -509,7 +525,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             if (r0 + r < nrhs) {
               const size_t e = ((size_t)(r0 + r) * nunits + y) * n2 + i;
               const float yr = sg * __uint_as_float(v[r]), yi = sg * __uint_as_float(v[NT + r]);
-              run.Y[e] = make_float2(yr, yi);
+              if (run.Yc) {
+                bool other = false;
+                double2 d = make_double2(f2d_fast(yr, other), f2d_fast(yi, other));
+                if (other) d = make_double2((double)yr, (double)yi);
+                run.Yc[e] = d;
+              } else {
+                run.Y[e] = make_float2(yr, yi);
+              }
               if (run.dotX) {
                 dre[r] += xq[r].x * yr + xq[r].y * yi;
                 dim[r] += xq[r].x * yi - xq[r].y * yr;
@@ -646,9 +669,10 @@ static mglma_status tc_grant_smem(size_t smem) {
   return MGLMA_OK;
 }
 
-template <int NT>
-static mglma_status launch_tc(mglma_ctx ctx, const mglma_coarse_s* C, const float2* X, float2* Y, int nrhs, int mode,
-                              void* xb, int* err, cudaStream_t s) {
+// X, Y: FP32 fields, or both canonical complex128
+template <int NT, typename E>
+static mglma_status launch_tc(mglma_ctx ctx, const mglma_coarse_s* C, const E* X, E* Y, int nrhs, int mode, void* xb,
+                              int* err, cudaStream_t s) {
   const int n2 = C->n2;
   const int64_t V1 = C->geo.V1;
   {
@@ -670,7 +694,8 @@ static mglma_status launch_tc(mglma_ctx ctx, const mglma_coarse_s* C, const floa
   run.dcount = nullptr;
   run.dout = nullptr;
   run.XB = run.XBself = (const uint8_t*)xb;
-  run.Y = Y;
+  run.Y = sizeof(E) == 8 ? (float2*)Y : nullptr;
+  run.Yc = sizeof(E) == 16 ? (double2*)Y : nullptr;
   run.d_lo = 0;
   run.d_hi = 8;
   run.par = -1;
@@ -727,6 +752,7 @@ static mglma_status launch_tc_eo(mglma_ctx ctx, const mglma_coarse_s* C, const f
   run.XB = xb_hop;
   run.XBself = xb_self;
   run.Y = Y;
+  run.Yc = nullptr;
   run.d_lo = d_lo;
   run.d_hi = d_hi;
   run.par = par;
@@ -837,7 +863,8 @@ mglma_status minres_flush(mglma_ctx ctx, const double* cf, int cap, const Vec& u
   return MGLMA_OK;
 }
 
-mglma_status coarse_apply_tc(mglma_ctx ctx, const mglma_coarse_s* C, const float2* X, float2* Y, int nrhs, int mode,
+template <typename E>
+static mglma_status apply_tc(mglma_ctx ctx, const mglma_coarse_s* C, const E* X, E* Y, int nrhs, int mode,
                              void* scratch, size_t scratch_bytes, cudaStream_t s) {
   if (!C->Aimg || !coarse_tc_supported(C->n2)) return fail(MGLMA_ERR_INVALID, "coarse_apply_tc: no tensor image");
   int* err = C->tc_err;
@@ -862,6 +889,18 @@ mglma_status coarse_apply_tc(mglma_ctx ctx, const mglma_coarse_s* C, const float
     st = launch_tc<8>(ctx, C, X, Y, nrhs, mode, xb, err, s);
   if (own) dfree(ctx, own, s);
   return st;
+}
+
+mglma_status coarse_apply_tc(mglma_ctx ctx, const mglma_coarse_s* C, const float2* X, float2* Y, int nrhs, int mode,
+                             void* scratch, size_t scratch_bytes, cudaStream_t s) {
+  return apply_tc(ctx, C, X, Y, nrhs, mode, scratch, scratch_bytes, s);
+}
+
+mglma_status coarse_apply_tc_canonical(mglma_ctx ctx, const mglma_coarse_s* C, const double* X, double* Y, int nrhs,
+                                       int mode, cudaStream_t s) {
+  const double V1 = (double)C->geo.V1, n2 = C->n2, N = nrhs;
+  ProfScope ps(ctx, K_COARSE, s, V1 * (9.0 * n2 * n2 * 4.0 + 2.0 * N * n2 * 16.0), V1 * 9.0 * n2 * n2 * 8.0 * N);
+  return apply_tc(ctx, C, (const double2*)X, (double2*)Y, nrhs, mode, nullptr, 0, s);
 }
 
 }  // namespace mglma

@@ -91,6 +91,10 @@ mglma_status coarse_tc_image(mglma_ctx ctx, mglma_coarse_s* C, cudaStream_t s);
 // allocated for the call (refused inside a graph capture)
 mglma_status coarse_apply_tc(mglma_ctx ctx, const mglma_coarse_s* C, const float2* X, float2* Y, int nrhs,
                              int mode, void* scratch, size_t scratch_bytes, cudaStream_t s);
+// the same between canonical complex128 fields on the device (Y may be X): values
+// rounded to FP32 on the way in, widened on the way out
+mglma_status coarse_apply_tc_canonical(mglma_ctx ctx, const mglma_coarse_s* C, const double* X, double* Y, int nrhs,
+                                       int mode, cudaStream_t s);
 size_t coarse_tc_scratch_bytes(const mglma_coarse_s* C, int nrhs);
 int coarse_tc_default_nt(int nrhs);
 mglma_status coarse_tc_check(mglma_coarse_s* C, cudaStream_t s);
