@@ -41,13 +41,6 @@ __device__ __forceinline__ double2 lc(double2 x, double2 y, double2 a, double2 b
   return o;
 }
 
-// a*x + y.  FP64 as four FMAs: the pipe is narrow enough that the eight products
-// of lc bound the vector updates (16 fields on 32x16^3: 830 us with lc)
-__device__ __forceinline__ float4 axy(float4 x, float4 y, double2 a) { return lc(x, y, a, make_double2(1, 0)); }
-__device__ __forceinline__ double2 axy(double2 x, double2 y, double2 a) {
-  return make_double2(fma(a.x, x.x, fma(-a.y, x.y, y.x)), fma(a.x, x.y, fma(a.y, x.x, y.y)));
-}
-
 // y_r = a_r x_r + b_r y_r (complex, per RHS; a NULL uses a_def, b NULL uses
 // b_def); sgn scales a.
 template <typename R>
@@ -72,11 +65,12 @@ __global__ void axpy2_kernel(const typename Pair<R>::T* p, typename Pair<R>::T* 
   const int r = blockIdx.y;
   const double2 ar = a[r];
   const double2 na = make_double2(-ar.x, -ar.y);
+  const double2 one = make_double2(1, 0);
   const size_t off = (size_t)r * m;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (size_t)gridDim.x * blockDim.x) {
     const auto pv = p[off + i], xv = x[off + i], wv = w[off + i], rv = res[off + i];
-    x[off + i] = axy(pv, xv, ar);
-    res[off + i] = axy(wv, rv, na);
+    x[off + i] = lc(pv, xv, ar, one);
+    res[off + i] = lc(wv, rv, na, one);
   }
 }
 
@@ -96,13 +90,14 @@ __global__ void multi_axpy_kernel(const typename Pair<R>::T* __restrict__ x0, ty
   }
   __syncthreads();
   const size_t off = (size_t)r * m;
+  const double2 one = make_double2(1, 0);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (size_t)gridDim.x * blockDim.x) {
     auto acc = y[off + i];
-    for (int j = 0; j < k; ++j) acc = axy(x0[j * jstride + off + i], acc, cs[j]);
+    for (int j = 0; j < k; ++j) acc = lc(x0[j * jstride + off + i], acc, cs[j], one);
     y[off + i] = acc;
     if (yb) {
       auto accb = yb[off + i];
-      for (int j = 0; j < k; ++j) accb = axy(x0b[j * jstride + off + i], accb, cs[j]);
+      for (int j = 0; j < k; ++j) accb = lc(x0b[j * jstride + off + i], accb, cs[j], one);
       yb[off + i] = accb;
     }
   }
@@ -233,11 +228,10 @@ struct RAcc<float> {
 template <>
 struct RAcc<double> {
   double N = 0, DR = 0, DI = 0;
-  // one FMA per product (see axy)
-  __device__ __forceinline__ void add_n(double2 a) { N = fma(a.x, a.x, fma(a.y, a.y, N)); }
+  __device__ __forceinline__ void add_n(double2 a) { N += a.x * a.x + a.y * a.y; }
   __device__ __forceinline__ void add_d(double2 a, double2 b) {
-    DR = fma(a.x, b.x, fma(a.y, b.y, DR));
-    DI = fma(a.x, b.y, fma(-a.y, b.x, DI));
+    DR += a.x * b.x + a.y * b.y;
+    DI += a.x * b.y - a.y * b.x;
   }
   __device__ __forceinline__ void add_nd(double2 a, double2 b) {
     add_n(a);
@@ -307,12 +301,13 @@ __global__ void __launch_bounds__(RT) axpy2_norm_kernel(const typename Pair<R>::
   const int r = blockIdx.y, nrhs = gridDim.y, nb = gridDim.x;
   const double2 ar = a[r];
   const double2 na = make_double2(-ar.x, -ar.y);
+  const double2 one = make_double2(1, 0);
   const size_t off = (size_t)r * m;
   RAcc<R> acc;
   for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < m; i += (size_t)nb * RT) {
     const auto pv = p[off + i], xv = x[off + i], wv = w[off + i], rv = res[off + i];
-    x[off + i] = axy(pv, xv, ar);
-    const auto nr = axy(wv, rv, na);
+    x[off + i] = lc(pv, xv, ar, one);
+    const auto nr = lc(wv, rv, na, one);
     res[off + i] = nr;
     acc.add_n(nr);
   }

@@ -48,55 +48,62 @@ __device__ __forceinline__ void minus_i_sigma(int k, double2 u0, double2 u1, dou
 constexpr int kChunk = 1024;  // sites per CTA
 
 // part[r][x0][chunk] = sum_k sum_{x in chunk of x0} <a[r][k-1](x), gamma5 gamma_k b[r](x)>,
-// times scale
+// times scale, on a grid of (L0 nc, nrhs); on (L0, nrhs) a CTA adds its slice's nc
+// chunks in the same order (no room for partial sums)
 __global__ void __launch_bounds__(256) contract_kernel(const double2* __restrict__ a, const double2* __restrict__ b,
-                                                       int64_t V, int64_t slice, double scale,
+                                                       int64_t V, int64_t slice, int nc, int L0, double scale,
                                                        double2* __restrict__ part) {
-  const int chunk = blockIdx.x, x0 = blockIdx.y, r = blockIdx.z;
-  const int64_t s0 = (int64_t)chunk * kChunk;
-  const int n = 3 * (int)min((int64_t)kChunk, slice - s0);
-  const int64_t site0 = (int64_t)x0 * slice + s0;
-  double sr = 0.0, si = 0.0;
-  for (int t = threadIdx.x; t < n; t += 256) {
-    const size_t e = (size_t)(site0 + t / 3) * 12 + t % 3;
-    double2 bv[4];
+  const int per = (int)gridDim.x / L0;  // CTAs per slice: nc or 1
+  const int x0 = blockIdx.x / per, r = blockIdx.y;
+  __shared__ double sh[8][2];
+  double2 sum = make_double2(0.0, 0.0);
+  for (int chunk = blockIdx.x % per; chunk < nc; chunk += per) {
+    const int64_t s0 = (int64_t)chunk * kChunk;
+    const int n = 3 * (int)min((int64_t)kChunk, slice - s0);
+    const int64_t site0 = (int64_t)x0 * slice + s0;
+    double sr = 0.0, si = 0.0;
+    for (int t = threadIdx.x; t < n; t += 256) {
+      const size_t e = (size_t)(site0 + t / 3) * 12 + t % 3;
+      double2 bv[4];
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) bv[sp] = __ldg(b + (size_t)r * V * 12 + e + 3 * sp);
+      for (int sp = 0; sp < 4; ++sp) bv[sp] = __ldg(b + (size_t)r * V * 12 + e + 3 * sp);
 #pragma unroll
-    for (int k = 1; k <= 3; ++k) {
-      const double2* ak = a + ((size_t)r * 3 + (k - 1)) * V * 12 + e;
-      double2 g[4];
-      minus_i_sigma(k, bv[2], bv[3], g[0], g[1]);  // upper = -i sigma_k b_lower
-      minus_i_sigma(k, bv[0], bv[1], g[2], g[3]);  // lower = -i sigma_k b_upper
+      for (int k = 1; k <= 3; ++k) {
+        const double2* ak = a + ((size_t)r * 3 + (k - 1)) * V * 12 + e;
+        double2 g[4];
+        minus_i_sigma(k, bv[2], bv[3], g[0], g[1]);  // upper = -i sigma_k b_lower
+        minus_i_sigma(k, bv[0], bv[1], g[2], g[3]);  // lower = -i sigma_k b_upper
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp) {
-        const double2 u = __ldg(ak + 3 * sp), w = g[sp];
-        sr = fma(u.x, w.x, sr);
-        sr = fma(u.y, w.y, sr);
-        si = fma(u.x, w.y, si);
-        si = fma(-u.y, w.x, si);
+        for (int sp = 0; sp < 4; ++sp) {
+          const double2 u = __ldg(ak + 3 * sp), w = g[sp];
+          sr = fma(u.x, w.x, sr);
+          sr = fma(u.y, w.y, sr);
+          si = fma(u.x, w.y, si);
+          si = fma(-u.y, w.x, si);
+        }
       }
     }
-  }
-  __shared__ double sh[8][2];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sr += __shfl_down_sync(0xffffffffu, sr, o);
-    si += __shfl_down_sync(0xffffffffu, si, o);
-  }
-  if (threadIdx.x % 32 == 0) {
-    sh[threadIdx.x / 32][0] = sr;
-    sh[threadIdx.x / 32][1] = si;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    sr = si = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      sr += sh[w][0];
-      si += sh[w][1];
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_down_sync(0xffffffffu, sr, o);
+      si += __shfl_down_sync(0xffffffffu, si, o);
     }
-    part[((size_t)r * gridDim.y + x0) * gridDim.x + chunk] = make_double2(scale * sr, scale * si);
+    if (threadIdx.x % 32 == 0) {
+      sh[threadIdx.x / 32][0] = sr;
+      sh[threadIdx.x / 32][1] = si;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      sr = si = 0.0;
+      for (int w = 0; w < 8; ++w) {
+        sr += sh[w][0];
+        si += sh[w][1];
+      }
+      sum = make_double2(sum.x + scale * sr, sum.y + scale * si);
+    }
+    __syncthreads();
   }
+  if (threadIdx.x == 0) part[(size_t)r * gridDim.x + blockIdx.x] = sum;
 }
 
 // out[i] = sum of the nc chunks of slice i
@@ -159,19 +166,24 @@ extern "C" mglma_status mglma_contract(mglma_ctx ctx, const mglma_lattice* lat, 
   MG_CHECK(stage_in(ctx, a, 3 * bb, s, ia));
   MG_CHECK(stage_in(ctx, b, bb, s, ib));
   MG_CHECK(stage_out_alloc(ctx, out, ob, s, o));
-  // one chunk per slice writes the result itself, more leave partial sums
-  const int nc = (int)((slice + kChunk - 1) / kChunk), nout = nrhs * lat->L[0];
+  // one CTA per slice writes the result itself, one per chunk leaves partial sums
+  const int nc = (int)((slice + kChunk - 1) / kChunk);
+  const int64_t nout = (int64_t)nrhs * lat->L[0], lim = (int64_t)1 << 31;
   double2* part = (double2*)o.dev;
-  if (nc > 1) MG_CHECK(dalloc(ctx, (void**)&part, (size_t)nout * nc * sizeof(double2), s));
+  bool split = nc > 1 && (int64_t)nc * lat->L[0] < lim && nout < lim;
+  if (split && dalloc(ctx, (void**)&part, (size_t)nout * nc * sizeof(double2), s) != MGLMA_OK) {
+    split = false;
+    part = (double2*)o.dev;
+  }
   {
     // algorithmic traffic: four spinors per site and RHS read once
     ProfScope ps(ctx, K_CONTRACT, s, 4.0 * (double)bb, 288.0 * (double)V * nrhs);
-    contract_kernel<<<dim3((unsigned)nc, (unsigned)lat->L[0], (unsigned)nrhs), 256, 0, s>>>(
-        (const double2*)ia.dev, (const double2*)ib.dev, V, slice, -1.0 / (3.0 * (double)slice), part);
-    if (nc > 1) contract_sum_kernel<<<(nout + 127) / 128, 128, 0, s>>>(part, nc, nout, (double2*)o.dev);
+    contract_kernel<<<dim3((unsigned)((split ? nc : 1) * lat->L[0]), (unsigned)nrhs), 256, 0, s>>>(
+        (const double2*)ia.dev, (const double2*)ib.dev, V, slice, nc, lat->L[0], -1.0 / (3.0 * (double)slice), part);
+    if (split) contract_sum_kernel<<<(unsigned)((nout + 127) / 128), 128, 0, s>>>(part, nc, (int)nout, (double2*)o.dev);
   }
   const cudaError_t launched = cudaGetLastError();
-  if (nc > 1) dfree(ctx, part, s);
+  if (split) dfree(ctx, part, s);
   MG_CUDA(launched);
   MG_CHECK(stage_out_finish(out, ob, s, o));
   return MGLMA_OK;

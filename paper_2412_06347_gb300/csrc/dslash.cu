@@ -236,24 +236,22 @@ __global__ void __launch_bounds__(128, dslash_min_ctas<R, NR, RW>()) dslash_kern
 #pragma unroll
     for (int r = 0; r < NR; ++r)
       if (r0 + r < a.nrhs && valid) {
-        {
-          if (a.g5out) {
+        if (a.g5out) {
 #pragma unroll
-            for (int k = 6; k < 12; ++k) acc[r][k] = -acc[r][k];
-          }
-          if (a.bsub) {
-            Cx<R> bv[12];
-            IO<R>::load(a.bsub, V, r0 + r, site, bv);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) acc[r][k] = bv[k] - acc[r][k];
-          }
-          if constexpr (BF) {
-            // the dots below see the values as stored
-#pragma unroll
-            for (int k = 0; k < 12; ++k) acc[r][k] = bf16_unpack(bf16_pack(acc[r][k]));
-          }
-          if constexpr (!CAN) SIO<SO>::store(out, V, r0 + r, site, acc[r]);
+          for (int k = 6; k < 12; ++k) acc[r][k] = -acc[r][k];
         }
+        if (a.bsub) {
+          Cx<R> bv[12];
+          IO<R>::load(a.bsub, V, r0 + r, site, bv);
+#pragma unroll
+          for (int k = 0; k < 12; ++k) acc[r][k] = bv[k] - acc[r][k];
+        }
+        if constexpr (BF) {
+          // the dots below see the values as stored
+#pragma unroll
+          for (int k = 0; k < 12; ++k) acc[r][k] = bf16_unpack(bf16_pack(acc[r][k]));
+        }
+        if constexpr (!CAN) SIO<SO>::store(out, V, r0 + r, site, acc[r]);
       }
     if constexpr (RED) {
       if (valid) {
@@ -1156,7 +1154,7 @@ mglma_status dslash(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& in, Spi
   return MGLMA_OK;
 }
 
-// FP64 on canonical spinors: four threads per site while that is what fills the
+// FP64 on canonical spinors: a warp per direction while that is what fills the
 // chip, see dslash_split_kernel
 static void launch_canon64(const mglma_gauge_s* G, const double* in, double* out, const DslashArgs& a, bool dagger,
                            cudaStream_t s) {

@@ -4,12 +4,21 @@
 // e = D^-1 (r / |r|) to a modest relative accuracy in FP32, x += |r| e, until
 // the FP64 residual reaches tol.  Inner FP32 flexible GCR(m) preconditioned by
 // the two-level correction of Sec. 2:
-//     z = T0 D1^-1 R0 r      (coarse solve: GCR on the stencil D1, BF16/FP32
-//                              operator, FP32 accumulation, loose tolerance)
-//     z += MR_nu(D, r - D z) (nu minimal-residual smoothing steps)
-// The pieces of Sec. 2: psi1 = T0 D1^-1 R0 b with D1^-1 solved to tol by a
-// coarse FP64 defect correction, psi0 = x - psi1 (App. chirality:
-// T Q1^-1 R gamma5 = T D1^-1 R when [P, gamma5] = 0).
+//     z = T0 D1^-1 R0 r      (coarse solve: MINRES or GCR on the stencil D1,
+//                              BF16/FP32 operator, FP32 accumulation, loose
+//                              tolerance)
+//     z += MR(D, r - D z)    (minimal-residual smoothing steps)
+// With every extent even the inner system is the even-odd one, S x_e = b' on
+// half-lattice fields (schur.cu), smoothed by (nu + 1) / 2 steps on S: a step on
+// S costs what one on D does and damps about what two do.  Steps on S against
+// the solve's time, 64x32^3, 16 RHS, to 1e-12, after the first version: 2 / 3 /
+// 4 / 5 / 7 -> 1192 / 1076 / 1158 / 1126 / 1271 ms (16 RHS of 32x16^3: 112 / 91 /
+// 81 / 81 / 80; one of 8^4: 26.6 / 20.1 / 17.7 / 15.5 / 12.6).  An odd extent
+// keeps the full system and nu steps on D.
+// The pieces of Sec. 2: psi1 = T0 D1^-1 R0 b with D1^-1 solved to tol by an
+// FP64 flexible GCR on the coarse operator (defect correction as a fallback),
+// psi0 = x - psi1 (App. chirality: T Q1^-1 R gamma5 = T D1^-1 R when [P, gamma5]
+// = 0).
 //
 // All RHS of a group advance together; every scalar is per RHS on the device
 // and converged RHS are frozen by device-side masks, so a RHS's iterates do
@@ -1312,8 +1321,21 @@ mglma_status coarse_solve64(mglma_ctx ctx, const mglma_coarse_s* C, const void* 
   MG_CHECK(zero_vec(ctx, vx, s));
   MG_CHECK(copy_vec(ctx, vb, vr, s));
   bool done = false;
-  MG_CHECK(coarse_fgcr64(ctx, C, vb, vx, vr, tol, &done, s));
+  const mglma_status fg = coarse_fgcr64(ctx, C, vb, vx, vr, tol, &done, s);
+  if (fg != MGLMA_ERR_OOM) MG_CHECK(fg);
   if (done) return C->Aimg ? coarse_tc_check(const_cast<mglma_coarse_s*>(C), s) : MGLMA_OK;
+  // go on from where it got to, or from X = 0 when it had no room for its basis
+  // or left a RHS worse than that
+  bool restart = fg == MGLMA_ERR_OOM;
+  if (!restart) {
+    MG_CHECK(norm2(ctx, vr, rr, s));
+    MG_CHECK(read_doubles(rr, hrr, n, s));
+    for (int i = 0; i < n; ++i) restart = restart || !(hrr[i] <= hbb[i]);
+  }
+  if (restart) {
+    MG_CHECK(zero_vec(ctx, vx, s));
+    MG_CHECK(copy_vec(ctx, vb, vr, s));
+  }
   OpFn Ac = [&](const Vec& in, Vec& out) { return coarse_apply(ctx, C, in.p, out.p, in.nrhs, MGLMA_FP32, CMODE_D, s); };
   const int tb = 64, nb = (n + tb - 1) / tb;
   for (int cycle = 0; cycle < 40; ++cycle) {
