@@ -49,7 +49,9 @@ constexpr int kChunk = 1024;  // sites per CTA
 
 // part[r][x0][chunk] = sum_k sum_{x in chunk of x0} <a[r][k-1](x), gamma5 gamma_k b[r](x)>,
 // times scale, on a grid of (L0 nc, nrhs); on (L0, nrhs) a CTA adds its slice's nc
-// chunks in the same order (no room for partial sums)
+// chunks in the same order (no room for partial sums, or a stream capture, whose
+// graph would own an allocation otherwise: the 48x24^3 case then takes the time of
+// one CTA per slice)
 __global__ void __launch_bounds__(256) contract_kernel(const double2* __restrict__ a, const double2* __restrict__ b,
                                                        int64_t V, int64_t slice, int nc, int L0, double scale,
                                                        double2* __restrict__ part) {
@@ -170,7 +172,9 @@ extern "C" mglma_status mglma_contract(mglma_ctx ctx, const mglma_lattice* lat, 
   const int nc = (int)((slice + kChunk - 1) / kChunk);
   const int64_t nout = (int64_t)nrhs * lat->L[0], lim = (int64_t)1 << 31;
   double2* part = (double2*)o.dev;
-  bool split = nc > 1 && (int64_t)nc * lat->L[0] < lim && nout < lim;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (nc > 1) MG_CUDA(cudaStreamIsCapturing(s, &cap));
+  bool split = nc > 1 && cap == cudaStreamCaptureStatusNone && (int64_t)nc * lat->L[0] < lim && nout < lim;
   if (split && dalloc(ctx, (void**)&part, (size_t)nout * nc * sizeof(double2), s) != MGLMA_OK) {
     split = false;
     part = (double2*)o.dev;
