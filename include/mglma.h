@@ -150,8 +150,8 @@ mglma_status mglma_dirac_apply(mglma_ctx ctx, mglma_gauge g, mglma_op op, int nr
  * device memory when they need the operator -- code running while a CUDA
  * graph is being captured, code called from inside an allocator hook, or a
  * process whose HBM is already fully reserved by another caching allocator.
- * It computes exactly what mglma_dirac_apply computes, but its two
- * internal-layout work fields live in one file-scope device array of 32 MiB
+ * It computes exactly what mglma_dirac_apply computes, but its work fields
+ * (none to two, by operator and precision) live in one file-scope device array of 32 MiB
  * that the library holds on every GPU that loads it, until the process
  * exits; the call makes no cudaMalloc/cudaFree and no allocating library call.
  *   in, out: DEVICE pointers to nrhs canonical spinors (host pointers are
@@ -163,7 +163,7 @@ mglma_status mglma_dirac_apply(mglma_ctx ctx, mglma_gauge g, mglma_op op, int nr
  *     (cudaGetSymbolAddress with that device current); make that first call
  *     before any stream capture.
  *   Every call shares the one array and leaves its last contents there;
- *     each call overwrites both work fields completely before reading them,
+ *     each call overwrites the work fields completely before reading them,
  *     so no clearing is needed.  Calls that overlap on the GPU (different
  *     streams, or different host threads) race on the array: serialise them. */
 mglma_status mglma_dirac_apply_noalloc(mglma_ctx ctx, mglma_gauge g, mglma_op op, int nrhs, const double* in,

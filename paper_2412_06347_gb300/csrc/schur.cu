@@ -21,13 +21,13 @@
 // pipe 50 %, issue slots 49 %, L1 51 %, DRAM 37 %, long-scoreboard stalls 4.5
 // of 7.7 warp cycles per instruction; 10 to 16 warps per SM measure the same.
 // The full-lattice stencil it replaces issued 2717 instructions per site and
-// RHS; here 1340.  Complex products run as packed FP32 pairs (one FFMA2 does
-// (re, im) with a duplicated link real, so a 3x3 complex product is 18 packed
-// FMAs plus 6 adds instead of 36 FMAs; duplicating the spinor's reals instead
-// measured 1788 against 1180 us), the links are stored as all 18 reals with
-// the time-boundary sign applied (no third row to rebuild, no hop factor: -1/2
-// rides on the stored inverse clover and on one packed FMA per component), and
-// links and clover are parity-split so a warp reads whole sectors.
+// RHS; the odd pass issues 1412.  Complex products run as packed FP32 pairs (one
+// FFMA2 does (re, im) with a duplicated link real, so a 3x3 complex product is 18
+// packed FMAs plus 6 adds instead of 36 FMAs; duplicating the spinor's reals
+// instead measured 1788 against 1180 us), the links are stored as all 18 reals
+// with the time-boundary sign applied (no third row to rebuild, no hop factor:
+// -1/2 rides on the stored inverse clover and on one packed FMA per component),
+// and links and clover are parity-split so a warp reads whole sectors.
 // 64x32^3, 16 RHS, us: odd pass BF16 1207 / FP32 1373, even pass MR step 1722,
 // dot 1470, FGCR image 1630; one MR step on S (2929) against 3500 for one on D
 // that damps about half as much.  A whole solve to 1e-12: 1507 -> 1102 ms.
