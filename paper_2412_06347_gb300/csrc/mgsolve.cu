@@ -334,14 +334,23 @@ static mglma_status gcr_run(GcrWork& w, const OpFn& A, const OpFn* M, const Vec&
     double* bb = w.sc.d + (size_t)(w.m + 1) * w.cap;
     std::vector<double> hb;
     MG_CHECK(read_doubles(bb, hb, n, s));
+    double* rr = w.sc.d + (size_t)w.m * w.cap;
+    MG_CUDA(cudaMemcpyAsync(rr, bb, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     // unit_ref: the reference is a residual of norm one of which b is a part
     for (int i = 0; i < n; ++i)
       hb[i] = (unit_ref ? (hb[i] > 0 ? 1.0 : 0.0) : hb[i]) * (*tol_scale)[i] * (*tol_scale)[i];
     MG_CUDA(cudaMemcpyAsync(bb, hb.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s));
+    // an RHS already at its target takes no step (it would take one whenever the
+    // others need one, and its result would depend on them)
+    gcr_mask_kernel<<<(n + 63) / 64, 64, 0, s>>>(rr, bb, tol * tol, w.sc.active, n);
+    MG_LAUNCH_CHECK();
     MG_CUDA(cudaStreamSynchronize(s));
   }
   std::vector<int> hact, prev;
-  if (poll_every == 1) MG_CHECK(read_active(w, n, prev));
+  if (poll_every == 1) {
+    MG_CHECK(read_active(w, n, prev));
+    if (std::none_of(prev.begin(), prev.end(), [](int a) { return a != 0; })) return MGLMA_OK;
+  }
   int it = 0;
   while (it < max_iter) {
     if (graphs && graphs->ready())
@@ -1216,6 +1225,14 @@ __global__ void masked_norm_kernel(const double* __restrict__ rr, const int* __r
   rinv[r] = v > 0 ? 1.0 / v : 0.0;
 }
 
+// RHS r0 .. r0 + n - 1 of a batch
+static Vec vsub(const Vec& v, int r0, int n) {
+  Vec o = v;
+  o.p = (char*)v.p + (size_t)r0 * v.n * (v.prec == MGLMA_FP64 ? 8 : 4);
+  o.nrhs = n;
+  return o;
+}
+
 // X (FP64 coarse, [n][V1][n2]) += D1^-1 (b1 - D1 X) towards |b1 - D1 X| <= tol |b1|:
 // FP64 flexible GCR on the FP64 operator, preconditioned by a loose FP32 coarse
 // solve on the stored operator (CoarseSolver: MINRES on g5hat S_ee on the tensor
@@ -1263,25 +1280,35 @@ static mglma_status coarse_fgcr64(mglma_ctx ctx, const mglma_coarse_s* C, const 
     MG_CHECK(cs.solve(r32, e32, inner, 240, &iters));
     return coarse_scale_convert(ctx, e32.p, MGLMA_FP32, z.p, MGLMA_FP64, rn, per, n, false, s);
   };
+  // An RHS whose residual is not finite or above |b1| is put back to X = 0 and
+  // left to the caller; each RHS goes its own way, whatever the others do.
   std::vector<double> hbb, hrr, scale(n);
+  std::vector<char> left(n, 0);
   MG_CHECK(norm2(ctx, vb, bb, s));
   MG_CHECK(read_doubles(bb, hbb, n, s));
-  for (int cycle = 0; cycle < 4; ++cycle) {
+  for (int cycle = 0;; ++cycle) {
     MG_CHECK(norm2(ctx, vr, rr, s));
     MG_CHECK(read_doubles(rr, hrr, n, s));
     bool any = false;
     for (int i = 0; i < n; ++i) {
       const double rel = hbb[i] > 0 ? std::sqrt(hrr[i] / hbb[i]) : 0.0;
-      if (!std::isfinite(rel)) return MGLMA_OK;  // left to the caller
-      any = any || rel > tol;
-      // reduction of this RHS's residual, relative to tol; one that is done
-      // starts inactive
-      scale[i] = rel > tol ? 0.5 / rel : 1.0 / tol;
+      if (!left[i] && !(rel <= 1)) {
+        left[i] = 1;
+        Vec xi = vsub(vx, i, 1), ri = vsub(vr, i, 1);
+        MG_CHECK(zero_vec(ctx, xi, s));
+        MG_CHECK(copy_vec(ctx, vsub(vb, i, 1), ri, s));
+      }
+      const bool go = !left[i] && rel > tol;
+      any = any || go;
+      // reduction of this RHS's residual, relative to tol; one that is done or
+      // left starts inactive
+      scale[i] = go ? 0.5 / rel : 2.0 / tol;
     }
     if (!any) {
-      *done = true;
+      *done = std::none_of(left.begin(), left.end(), [](char l) { return l != 0; });
       return MGLMA_OK;
     }
+    if (cycle == 4) return MGLMA_OK;
     GcrResult gr;
     MG_CHECK(gcr_run(w, A, &M, vr, ve, 60, tol, 1, gr, &scale, nullptr));
     MG_CHECK(axpby(ctx, nullptr, C1, ve, nullptr, C1, vx, s));  // X += e ; r = b1 - D1 X
@@ -1289,7 +1316,6 @@ static mglma_status coarse_fgcr64(mglma_ctx ctx, const mglma_coarse_s* C, const 
     MG_CHECK(copy_vec(ctx, vb, vr, s));
     MG_CHECK(axpby(ctx, nullptr, CM1, ve, nullptr, C1, vr, s));
   }
-  return MGLMA_OK;
 }
 
 // X (FP64 coarse, [n][V1][n2]) = D1^-1 b1 to tol: flexible GCR as above, and FP64
@@ -1326,15 +1352,8 @@ mglma_status coarse_solve64(mglma_ctx ctx, const mglma_coarse_s* C, const void* 
   const mglma_status fg = coarse_fgcr64(ctx, C, vb, vx, vr, tol, &done, s);
   if (fg != MGLMA_ERR_OOM) MG_CHECK(fg);
   if (done) return C->Aimg ? coarse_tc_check(const_cast<mglma_coarse_s*>(C), s) : MGLMA_OK;
-  // go on from where it got to, or from X = 0 when it had no room for its basis
-  // or left a RHS worse than that
-  bool restart = fg == MGLMA_ERR_OOM;
-  if (!restart) {
-    MG_CHECK(norm2(ctx, vr, rr, s));
-    MG_CHECK(read_doubles(rr, hrr, n, s));
-    for (int i = 0; i < n; ++i) restart = restart || !(hrr[i] <= hbb[i]);
-  }
-  if (restart) {
+  // go on from where it got to, or from X = 0 when it had no room
+  if (fg == MGLMA_ERR_OOM) {
     MG_CHECK(zero_vec(ctx, vx, s));
     MG_CHECK(copy_vec(ctx, vb, vr, s));
   }
@@ -1376,12 +1395,6 @@ mglma_status coarse_solve64(mglma_ctx ctx, const mglma_coarse_s* C, const void* 
 // FP64 tolerance leaves.  Every RHS follows exactly the recurrence it would
 // follow alone (its own scalars, masks and restart points), so its result
 // does not depend on what else is in flight.
-static Vec vsub(const Vec& v, int r0, int n) {
-  Vec o = v;
-  o.p = (char*)v.p + (size_t)r0 * v.n * (v.prec == MGLMA_FP64 ? 8 : 4);
-  o.nrhs = n;
-  return o;
-}
 static Spinor ssub(const Spinor& v, int r0, int n) {
   Spinor o = v;
   o.p = (char*)v.p + (size_t)r0 * v.rhs_reals() * (v.prec == MGLMA_FP64 ? 8 : 4);
