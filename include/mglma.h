@@ -138,6 +138,7 @@ mglma_status mglma_gauge_info(mglma_gauge g, int L[4], int64_t* volume);
  * arithmetic: MGLMA_FP64 (FP64 links and clover) or MGLMA_FP32 (FP32
  * reconstruct-12 links, FP32 clover, inputs rounded to FP32).  The definition
  * of D is the one stated at the top of this header (Sec. 2: Q = gamma5 D).
+ * A RHS's result is the same bits whatever nrhs is.
  * MGLMA_OP_SCHUR / _SCHUR_Q (FP64 only, every extent even): the even-odd
  * operator S (or gamma5 S) reads the even sites of in and writes the even
  * sites of out, zero on the odd ones; the first call on a gauge field forms

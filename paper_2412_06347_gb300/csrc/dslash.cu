@@ -637,28 +637,46 @@ __global__ void __launch_bounds__(128) dslash_slot_kernel(const double2* __restr
 
 // ------------------------------------------------------------ FP64 stencil, four threads per site
 // Few sites: D (or D^dag) on canonical complex128 spinors, a CTA of four warps
-// per 32 sites of one RHS.  Warp mu takes the two hops of direction mu; the sums
-// meet in shared memory, and warp mu adds rows 3 mu .. 3 mu + 2 of the clover
-// term and writes those components.  With one thread per site an 8^4 spinor is
-// 128 warps, one per SM at most, each alone with its SM's FP64 pipe.
+// per 32 sites of one RHS.  Warp mu takes the two hops of direction mu as far as
+// their half spinors, which meet in shared memory; warp mu then forms the three
+// components of spin mu: the rows of the clover term plus the eight hops in the
+// order of dslash_kernel, operation by operation, so a RHS gets the same bits
+// from both kernels, alone and in any batch.  With one thread per site an 8^4
+// spinor is 128 warps, one per SM at most, each alone with its SM's FP64 pipe.
 template <bool DAG, int MU>
 __device__ __forceinline__ void split_hops(const double2* in, const double2* U, const DslashArgs& a, int r,
-                                           int64_t site, const int x[4], Cx<double> acc[12]) {
+                                           int64_t site, const int x[4], double2 (*sh)[6][32], int lane) {
   const double sF = DAG ? 1.0 : -1.0;
   const int64_t V = a.q.V, nf = nbr_fwd(a.q, site, x, MU), nb = nbr_bwd(a.q, site, x, MU);
   const double ff = -0.5 * ((MU == 0 && x[0] == a.q.L[0] - 1) ? a.bc : 1.0);
   const double fb = -0.5 * ((MU == 0 && x[0] == 0) ? a.bc : 1.0);
-  Cx<double> psi[12];
+  Cx<double> psi[12], g[6];
   M3<double> Um;
   Link<double>::load(U, V, MU, site, Um);
   SIO<Canon64>::load(in, V, r, nf, psi);
-  hop_add<double, true>(MU, sF, ff, Um, psi, acc);
+  hop_half<double, true>(MU, sF, ff, Um, psi, g, g + 3);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) sh[2 * MU][k][lane] = make_double2(g[k].re, g[k].im);
   Link<double>::load(U, V, MU, nb, Um);
   SIO<Canon64>::load(in, V, r, nb, psi);
-  hop_add<double, false>(MU, -sF, fb, Um, psi, acc);
+  hop_half<double, false>(MU, -sF, fb, Um, psi, g, g + 3);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) sh[2 * MU + 1][k][lane] = make_double2(g[k].re, g[k].im);
 }
 
-// o[k] += row 3 HALF + k of the packed Hermitian block times v
+// component (SP, c) of the hop in direction MU with sign s from its half spinor
+// (see reconstruct_add)
+template <int SP, int MU>
+__device__ __forceinline__ Cx<double> split_part(double s, const double2 (*g)[32], int c, int lane) {
+  constexpr bool exch = SP >= 2 && (MU == 1 || MU == 2);
+  const double2 v = g[3 * ((SP & 1) ^ (exch ? 1 : 0)) + c][lane];
+  const Cx<double> h = cx(v.x, v.y);
+  if (SP < 2) return h;
+  const Cx<double> t = MU == 1 || MU == 3 ? mul_i(h) : h;
+  return MU == 0 || (SP == 3 && MU >= 2) ? -(s * t) : s * t;
+}
+
+// rows 3 HALF .. 3 HALF + 2 of the packed Hermitian block times v (as clover_apply6)
 template <int HALF>
 __device__ __forceinline__ void split_clover(const double c[36], const Cx<double> v[6], Cx<double> o[3]) {
 #pragma unroll
@@ -674,7 +692,24 @@ __device__ __forceinline__ void split_clover(const double c[36], const Cx<double
       else
         cfma_conj(s, cx(c[e], c[e + 1]), v[j]);
     }
-    o[k] = o[k] + s;
+    o[k] = s;
+  }
+}
+
+// o += the eight hops' spin SP
+template <bool DAG, int SP>
+__device__ __forceinline__ void split_sum(const double2 (*sh)[6][32], int lane, Cx<double> o[3]) {
+  const double sF = DAG ? 1.0 : -1.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    o[k] = o[k] + split_part<SP, 0>(sF, sh[0], k, lane);
+    o[k] = o[k] + split_part<SP, 0>(-sF, sh[1], k, lane);
+    o[k] = o[k] + split_part<SP, 1>(sF, sh[2], k, lane);
+    o[k] = o[k] + split_part<SP, 1>(-sF, sh[3], k, lane);
+    o[k] = o[k] + split_part<SP, 2>(sF, sh[4], k, lane);
+    o[k] = o[k] + split_part<SP, 2>(-sF, sh[5], k, lane);
+    o[k] = o[k] + split_part<SP, 3>(sF, sh[6], k, lane);
+    o[k] = o[k] + split_part<SP, 3>(-sF, sh[7], k, lane);
   }
 }
 
@@ -682,23 +717,18 @@ template <bool DAG>
 __global__ void __launch_bounds__(128) dslash_split_kernel(const double2* __restrict__ in, double2* __restrict__ out,
                                                            const double2* __restrict__ U, const double2* __restrict__ C,
                                                            DslashArgs a) {
-  __shared__ double2 sh[4][12][32];
+  __shared__ double2 sh[8][6][32];
   const int64_t V = a.q.V;
   const int mu = threadIdx.x / 32, lane = threadIdx.x % 32, r = blockIdx.y;
   const int64_t site0 = (int64_t)blockIdx.x * 32 + lane, site = site0 < V ? site0 : V - 1;
   int x[4];
   site_coords(a.q, site, x);
-  Cx<double> acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = cx(0.0, 0.0);
   switch (mu) {
-    case 0: split_hops<DAG, 0>(in, U, a, r, site, x, acc); break;
-    case 1: split_hops<DAG, 1>(in, U, a, r, site, x, acc); break;
-    case 2: split_hops<DAG, 2>(in, U, a, r, site, x, acc); break;
-    default: split_hops<DAG, 3>(in, U, a, r, site, x, acc); break;
+    case 0: split_hops<DAG, 0>(in, U, a, r, site, x, sh, lane); break;
+    case 1: split_hops<DAG, 1>(in, U, a, r, site, x, sh, lane); break;
+    case 2: split_hops<DAG, 2>(in, U, a, r, site, x, sh, lane); break;
+    default: split_hops<DAG, 3>(in, U, a, r, site, x, sh, lane); break;
   }
-#pragma unroll
-  for (int k = 0; k < 12; ++k) sh[mu][k][lane] = make_double2(acc[k].re, acc[k].im);
   const int chi = mu / 2;
   double c[36];
   Clover<double>::load(C, V, chi, site, c);
@@ -709,20 +739,17 @@ __global__ void __launch_bounds__(128) dslash_split_kernel(const double2* __rest
     const double2 q = __ldg(p + k);
     v[k] = cx(q.x, q.y);
   }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    o[k] = cx(0.0, 0.0);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const double2 q = sh[m][3 * mu + k][lane];
-      o[k] = o[k] + cx(q.x, q.y);
-    }
-  }
   if (mu & 1)
     split_clover<1>(c, v, o);
   else
     split_clover<0>(c, v, o);
+  __syncthreads();
+  switch (mu) {
+    case 0: split_sum<DAG, 0>(sh, lane, o); break;
+    case 1: split_sum<DAG, 1>(sh, lane, o); break;
+    case 2: split_sum<DAG, 2>(sh, lane, o); break;
+    default: split_sum<DAG, 3>(sh, lane, o); break;
+  }
   if (site0 >= V) return;
   const double g = a.g5out && chi ? -1.0 : 1.0;
   double2* w = out + ((size_t)r * V + site) * 12 + 3 * mu;
@@ -1058,7 +1085,8 @@ static double dslash_bytes(int64_t V, int nrhs, bool fp64) {
 static double dslash_flops(int64_t V, int nrhs) { return 1896.0 * (double)V * nrhs; }
 
 // site-RHS products up to which the FP64 stencil on canonical fields takes four
-// threads per site: 4096 sites 16.6 against 43.4 us with one thread per site,
+// threads per site: 4096 sites 16.4 against 43.4 us with one thread per site (16.1
+// when the directions' sums were added instead of the hops in order),
 // 16384 47.5 against 43.4 (one warp on each quarter of 128 SMs by then), 65536
 // the same
 constexpr size_t kSplitSites = 12288;

@@ -316,10 +316,12 @@ __device__ __forceinline__ void mat_dag_vec(const M3<R>& U, const Cx<R> h[3], Cx
   }
 }
 
-// one hop term: acc += f * (1 + s gamma_mu) W psi, W = U (fwd) or U^dag (bwd)
+// upper half (g0, g1) of one hop term f * (1 + s gamma_mu) W psi, W = U (fwd) or
+// U^dag (bwd); reconstruct_add gives both halves
 template <typename R, bool FWD>
-__device__ __forceinline__ void hop_add(int mu, R s, R f, const M3<R>& U, const Cx<R> psi[12], Cx<R> acc[12]) {
-  Cx<R> h0[3], h1[3], g0[3], g1[3];
+__device__ __forceinline__ void hop_half(int mu, R s, R f, const M3<R>& U, const Cx<R> psi[12], Cx<R> g0[3],
+                                         Cx<R> g1[3]) {
+  Cx<R> h0[3], h1[3];
   project<R>(mu, s, psi, h0, h1);
   if (FWD) {
     mat_vec<R>(U, h0, g0);
@@ -333,6 +335,13 @@ __device__ __forceinline__ void hop_add(int mu, R s, R f, const M3<R>& U, const 
     g0[c] = f * g0[c];
     g1[c] = f * g1[c];
   }
+}
+
+// one hop term: acc += f * (1 + s gamma_mu) W psi
+template <typename R, bool FWD>
+__device__ __forceinline__ void hop_add(int mu, R s, R f, const M3<R>& U, const Cx<R> psi[12], Cx<R> acc[12]) {
+  Cx<R> g0[3], g1[3];
+  hop_half<R, FWD>(mu, s, f, U, psi, g0, g1);
   reconstruct_add<R>(mu, s, g0, g1, acc);
 }
 
