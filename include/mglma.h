@@ -379,8 +379,10 @@ mglma_status mglma_sources(mglma_ctx ctx, const mglma_lattice* lat, int kind, in
  * sources are mglma_gamma5_gamma of eta).
  *   a: nrhs x 3 canonical spinors ([r][k-1][site][spin][colour]);
  *   b: nrhs canonical spinors; out: nrhs x L0 complex128 ([r][x0]).
- * Host or device pointers.  Sums in FP64 in a fixed order (one CTA per RHS
- * and time slice), so the result does not depend on the batch. */
+ * Host or device pointers.  Sums in FP64 in a fixed order (chunks of 1024
+ * sites of one RHS and time slice, the chunks in order), so the result does not
+ * depend on the batch, nor on whether the call is captured or finds no room for
+ * the chunks' sums (the chunks of a slice then run one after the other). */
 mglma_status mglma_contract(mglma_ctx ctx, const mglma_lattice* lat, int nrhs, const double* a, const double* b,
                             double* out, void* cuda_stream);
 /* out = gamma5 gamma_k in for nrhs canonical spinors, k = 1, 2, 3 (chiral

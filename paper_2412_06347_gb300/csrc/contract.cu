@@ -101,7 +101,9 @@ __global__ void __launch_bounds__(256) contract_kernel(const double2* __restrict
         sr += sh[w][0];
         si += sh[w][1];
       }
-      sum = make_double2(sum.x + scale * sr, sum.y + scale * si);
+      // product and sum rounded separately, as when contract_sum_kernel adds the
+      // chunks: both grids give the same bits
+      sum = make_double2(__dadd_rn(sum.x, __dmul_rn(scale, sr)), __dadd_rn(sum.y, __dmul_rn(scale, si)));
     }
     __syncthreads();
   }
