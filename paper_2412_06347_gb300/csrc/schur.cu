@@ -441,10 +441,11 @@ struct EvArgs {
   const void* r = nullptr;
 };
 
-// per-thread partials summed over the CTA's warp in FP32 (the FP64 pipe of GB300
-// is too narrow for a per-thread FP64 tree), written as FP64
+// per-thread sums of one site each added over the CTA's warp in FP32 (the FP64 pipe
+// of GB300 is too narrow for a per-thread FP64 tree) and to acc in FP64: FP32
+// never carries more than the 32 sites of a warp, whatever nsub is
 template <int NV>
-__device__ __forceinline__ void warp_partials(float* v, double* dst) {
+__device__ __forceinline__ void warp_partials(float* v, double* acc) {
   static_assert(SCHUR_T == 32, "one warp per CTA");
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -452,7 +453,7 @@ __device__ __forceinline__ void warp_partials(float* v, double* dst) {
     for (int e = 0; e < NV; ++e) v[e] += __shfl_down_sync(0xffffffffu, v[e], o);
   if (threadIdx.x == 0)
 #pragma unroll
-    for (int e = 0; e < NV; ++e) dst[e] = (double)v[e];
+    for (int e = 0; e < NV; ++e) acc[e] += (double)v[e];
 }
 
 template <int EV>
@@ -465,110 +466,120 @@ __global__ void __launch_bounds__(SCHUR_T, schur_ctas<EV>())
   using SX = typename std::conditional<BFX, SpinBf16, float>::type;
   const EoTile t(g, nrhs);
   const int r = t.r;
-  float v[NV];
+  __shared__ double sum[NV];  // thread 0's
+  if (RED && threadIdx.x == 0)
 #pragma unroll
-  for (int e = 0; e < NV; ++e) v[e] = 0.f;
+    for (int e = 0; e < NV; ++e) sum[e] = 0.0;
   for (int k = 0; k < nsub; ++k) {
-    const uint32_t u = (t.blk * nsub + k) * SCHUR_T + threadIdx.x;
-    if (u >= g.Vh) break;
-    float2 acc[12];
-    hops2<float>(g, u, 0, U, rhs_of<float>(w, g, r), acc);
-    if (EV == EV_PREP) {
-      Sp<float> q;
-      q.load(rhs_of<float>(a.b, g, r), g.Vh, u);
+    const uint32_t u0 = (t.blk * nsub + k) * SCHUR_T, u = u0 + threadIdx.x;
+    if (u0 >= g.Vh) break;
+    float v[NV];
 #pragma unroll
-      for (int j = 0; j < 12; ++j) acc[j] = fma2(acc[j], dup(0.5f), q.get(j));
-    } else {  // S x = A x + hops / 2
-      Sp<SX> q;
-      q.load(rhs_of<SX>(x, g, r), g.Vh, u);
-      float2 p[12];
+    for (int e = 0; e < NV; ++e) v[e] = 0.f;
+    if (u < g.Vh) {
+      float2 acc[12];
+      hops2<float>(g, u, 0, U, rhs_of<float>(w, g, r), acc);
+      if (EV == EV_PREP) {
+        Sp<float> q;
+        q.load(rhs_of<float>(a.b, g, r), g.Vh, u);
 #pragma unroll
-      for (int j = 0; j < 12; ++j) p[j] = q.get(j);
+        for (int j = 0; j < 12; ++j) acc[j] = fma2(acc[j], dup(0.5f), q.get(j));
+      } else {  // S x = A x + hops / 2
+        Sp<SX> q;
+        q.load(rhs_of<SX>(x, g, r), g.Vh, u);
+        float2 p[12];
 #pragma unroll
-      for (int chi = 0; chi < 2; ++chi) {
-        float c[36];
-        float2 o[6];
-        clover_load2(C, g.Vh, chi, u, c);
-        clover2(c, p + 6 * chi, o);
+        for (int j = 0; j < 12; ++j) p[j] = q.get(j);
 #pragma unroll
-        for (int j = 0; j < 6; ++j) acc[6 * chi + j] = fma2(acc[6 * chi + j], dup(0.5f), o[j]);
-      }
-    }
-    if (EV == EV_PREP || EV == EV_APPLY) {
-      Sp<float>::store(rhs_of<float>(out, g, r), g.Vh, u, acc);
-    } else if (EV == EV_RES) {
-      Sp<float> q;
-      q.load(rhs_of<float>(a.b, g, r), g.Vh, u);
+        for (int chi = 0; chi < 2; ++chi) {
+          float c[36];
+          float2 o[6];
+          clover_load2(C, g.Vh, chi, u, c);
+          clover2(c, p + 6 * chi, o);
 #pragma unroll
-      for (int j = 0; j < 12; ++j) acc[j] = adds<-1>(q.get(j), acc[j]);
-      Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
-    } else if (EV == EV_DOT) {
-      Sp<SpinBf16> p;
-      p.load(rhs_of<SpinBf16>(x, g, r), g.Vh, u);
-#pragma unroll
-      for (int j = 0; j < 12; ++j) {
-        const float2 q = unpack2(pack2(acc[j])), y = p.get(j);  // the dots see the values as stored
-        acc[j] = q;
-        v[0] += q.x * q.x + q.y * q.y;
-        v[1] += q.x * y.x + q.y * y.y;
-        v[2] += q.x * y.y - q.y * y.x;
-      }
-      Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
-    } else if (EV == EV_MR) {
-      const float2 al = a.alpha[r];
-      // complex -a v = nr (re, im) + ni (im, re) with ni = (Im a, -Im a)
-      const float2 nr = dup(-al.x), ni = make_float2(al.y, -al.y);
-      const char *tp = rhs_of<SpinBf16>(x, g, r), *sp = rhs_of<SpinBf16>(a.s, g, r);
-      char *op = rhs_of<SpinBf16>(out, g, r), *np = rhs_of<SpinBf16>(a.sn, g, r);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const uint4 tv = ldg_row<uint4>(tp, g.Vh, j, u), sv = ldg_row<uint4>(sp, g.Vh, j, u);
-        const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w}, sw[4] = {sv.x, sv.y, sv.z, sv.w};
-        uint32_t to[4], so[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const float2 tk = unpack2(tw[h]), sk = unpack2(sw[h]), q = acc[4 * j + h];
-          to[h] = pack2(fma2(ni, make_float2(q.y, q.x), fma2(nr, q, tk)));
-          so[h] = pack2(fma2(ni, make_float2(tk.y, tk.x), fma2(nr, tk, sk)));
-          const float2 tn = unpack2(to[h]), sn = unpack2(so[h]);
-          v[0] += tn.x * tn.x + tn.y * tn.y;
-          v[1] += tn.x * sn.x + tn.y * sn.y;
-          v[2] += tn.x * sn.y - tn.y * sn.x;
+          for (int j = 0; j < 6; ++j) acc[6 * chi + j] = fma2(acc[6 * chi + j], dup(0.5f), o[j]);
         }
-        row<uint4>(op, g.Vh, j, u) = make_uint4(to[0], to[1], to[2], to[3]);
-        row<uint4>(np, g.Vh, j, u) = make_uint4(so[0], so[1], so[2], so[3]);
       }
-    } else {
-      Sp<float>::store(rhs_of<float>(out, g, r), g.Vh, u, acc);
-      if (a.k == 0) {
-        const char* rp = rhs_of<float>(a.r, g, r);
+      if (EV == EV_PREP || EV == EV_APPLY) {
+        Sp<float>::store(rhs_of<float>(out, g, r), g.Vh, u, acc);
+      } else if (EV == EV_RES) {
+        Sp<float> q;
+        q.load(rhs_of<float>(a.b, g, r), g.Vh, u);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          const float4 q = ldg_row<float4>(rp, g.Vh, c, u);
-          const float2 w0 = acc[2 * c], w1 = acc[2 * c + 1];
-          v[0] += w0.x * w0.x + w0.y * w0.y + w1.x * w1.x + w1.y * w1.y;
-          v[1] += w0.x * q.x + w0.y * q.y + w1.x * q.z + w1.y * q.w;
-          v[2] += w0.x * q.y - w0.y * q.x + w1.x * q.w - w1.y * q.z;
+        for (int j = 0; j < 12; ++j) acc[j] = adds<-1>(q.get(j), acc[j]);
+        Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
+      } else if (EV == EV_DOT) {
+        Sp<SpinBf16> p;
+        p.load(rhs_of<SpinBf16>(x, g, r), g.Vh, u);
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+          const float2 q = unpack2(pack2(acc[j])), y = p.get(j);  // the dots see the values as stored
+          acc[j] = q;
+          v[0] += q.x * q.x + q.y * q.y;
+          v[1] += q.x * y.x + q.y * y.y;
+          v[2] += q.x * y.y - q.y * y.x;
         }
-      } else {
+        Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
+      } else if (EV == EV_MR) {
+        const float2 al = a.alpha[r];
+        // complex -a v = nr (re, im) + ni (im, re) with ni = (Im a, -Im a)
+        const float2 nr = dup(-al.x), ni = make_float2(al.y, -al.y);
+        const char *tp = rhs_of<SpinBf16>(x, g, r), *sp = rhs_of<SpinBf16>(a.s, g, r);
+        char *op = rhs_of<SpinBf16>(out, g, r), *np = rhs_of<SpinBf16>(a.sn, g, r);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          if (j >= a.k) break;
-          const char* wp = rhs_of<float>((const void*)(a.W0 + j * a.wslot), g, r);
+          const uint4 tv = ldg_row<uint4>(tp, g.Vh, j, u), sv = ldg_row<uint4>(sp, g.Vh, j, u);
+          const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w}, sw[4] = {sv.x, sv.y, sv.z, sv.w};
+          uint32_t to[4], so[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const float2 tk = unpack2(tw[h]), sk = unpack2(sw[h]), q = acc[4 * j + h];
+            to[h] = pack2(fma2(ni, make_float2(q.y, q.x), fma2(nr, q, tk)));
+            so[h] = pack2(fma2(ni, make_float2(tk.y, tk.x), fma2(nr, tk, sk)));
+            const float2 tn = unpack2(to[h]), sn = unpack2(so[h]);
+            v[0] += tn.x * tn.x + tn.y * tn.y;
+            v[1] += tn.x * sn.x + tn.y * sn.y;
+            v[2] += tn.x * sn.y - tn.y * sn.x;
+          }
+          row<uint4>(op, g.Vh, j, u) = make_uint4(to[0], to[1], to[2], to[3]);
+          row<uint4>(np, g.Vh, j, u) = make_uint4(so[0], so[1], so[2], so[3]);
+        }
+      } else {
+        Sp<float>::store(rhs_of<float>(out, g, r), g.Vh, u, acc);
+        if (a.k == 0) {
+          const char* rp = rhs_of<float>(a.r, g, r);
 #pragma unroll
           for (int c = 0; c < 6; ++c) {
-            const float4 q = ldg_row<float4>(wp, g.Vh, c, u);
+            const float4 q = ldg_row<float4>(rp, g.Vh, c, u);
             const float2 w0 = acc[2 * c], w1 = acc[2 * c + 1];
-            v[(2 * j) % NV] += q.x * w0.x + q.y * w0.y + q.z * w1.x + q.w * w1.y;
-            v[(2 * j + 1) % NV] += q.x * w0.y - q.y * w0.x + q.z * w1.y - q.w * w1.x;
+            v[0] += w0.x * w0.x + w0.y * w0.y + w1.x * w1.x + w1.y * w1.y;
+            v[1] += w0.x * q.x + w0.y * q.y + w1.x * q.z + w1.y * q.w;
+            v[2] += w0.x * q.y - w0.y * q.x + w1.x * q.w - w1.y * q.z;
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            if (j >= a.k) break;
+            const char* wp = rhs_of<float>((const void*)(a.W0 + j * a.wslot), g, r);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+              const float4 q = ldg_row<float4>(wp, g.Vh, c, u);
+              const float2 w0 = acc[2 * c], w1 = acc[2 * c + 1];
+              v[(2 * j) % NV] += q.x * w0.x + q.y * w0.y + q.z * w1.x + q.w * w1.y;
+              v[(2 * j + 1) % NV] += q.x * w0.y - q.y * w0.x + q.z * w1.y - q.w * w1.x;
+            }
           }
         }
       }
     }
+    if (RED) {
+      __syncwarp();
+      warp_partials<NV>(v, sum);
+    }
   }
   if (RED) {
     __syncwarp();
-    warp_partials<NV>(v, a.part + ((size_t)r * eo_blocks(g.Vh) + t.blk) * NV);
+    if (threadIdx.x < NV) a.part[((size_t)r * eo_blocks(g.Vh) + t.blk) * NV + threadIdx.x] = sum[threadIdx.x];
   }
 }
 
