@@ -565,7 +565,9 @@ mglma_status mglma_serve(mglma_ctx ctx, const mglma_serve_config* cfg, mglma_req
  *     with RW = 1); or the staged-tile kernel, 32 sites x NRT RHS per CTA
  *     with each site's links and clover staged once in shared memory, coded
  *     64 + NRT (NRT = 4, 8, 16);
- *   kernel 1: RHS per tile of the tensor-core coarse stencil (8, 16, 32), needs c.
+ *   kernel 1: RHS per tile of the tensor-core coarse stencil (8, 16, 32), needs c;
+ *     applications of the full operator only (the even-odd ones of the default
+ *     coarse solver take all RHS in one tile up to 32).
  * g or c may be NULL to skip that kernel. */
 mglma_status mglma_autotune(mglma_ctx ctx, mglma_gauge g, mglma_coarse c, int nrhs);
 /* Sets the choice for kernel / the RHS bucket of nrhs by hand (codes as

@@ -344,15 +344,14 @@ static mglma_status schur_composed(mglma_ctx ctx, const mglma_coarse_s* C, const
   return MGLMA_OK;
 }
 
-bool coarse_schur_dot_ok(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs, int prec) {
-  return prec == MGLMA_FP32 && C->Aimg && C->Sinv_img && C->tc_dpart && nrhs >= 1 &&
-         nrhs <= tuned(ctx, TUNE_COARSE_NT, nrhs, C->geo.V1, coarse_tc_default_nt(nrhs));
+bool coarse_schur_dot_ok(const mglma_coarse_s* C, int nrhs, int prec) {
+  return prec == MGLMA_FP32 && C->Aimg && C->Sinv_img && C->tc_dpart && nrhs >= 1 && nrhs <= coarse_eo_nt(nrhs);
 }
 
 mglma_status coarse_schur_apply(mglma_ctx ctx, const mglma_coarse_s* C, const void* Xe, void* Ye, int nrhs, int prec,
                                 int mode, void* scratch, size_t scratch_bytes, cudaStream_t s, double2* dot_out,
                                 bool x_imaged) {
-  if (dot_out && !coarse_schur_dot_ok(ctx, C, nrhs, prec))
+  if (dot_out && !coarse_schur_dot_ok(C, nrhs, prec))
     return fail(MGLMA_ERR_INVALID, "schur apply: the fused dot needs the tensor-core path and one RHS tile");
   if (x_imaged && !dot_out) return fail(MGLMA_ERR_INVALID, "schur apply: a given X image goes with the fused dot");
   if (!C->Sinv64 && !C->Sinv_img) return fail(MGLMA_ERR_INVALID, "schur apply: even-odd set-up missing");

@@ -769,12 +769,12 @@ mglma_status coarse_tc_eo_launch(mglma_ctx ctx, const mglma_coarse_s* C, const f
                                  const uint16_t* Ahop, const float2* dotX, double2* dot_out, bool hop_imaged) {
   if (!C->Aimg || !coarse_tc_supported(C->n2)) return fail(MGLMA_ERR_INVALID, "coarse_tc_eo: no tensor image");
   if (hop_imaged && (mode & 1)) return fail(MGLMA_ERR_INVALID, "coarse_tc_eo: a given hop image carries no gamma5hat");
-  if (dot_out && (!dotX || !C->tc_dpart || nrhs > tuned(ctx, TUNE_COARSE_NT, nrhs, C->geo.V1, coarse_tc_default_nt(nrhs))))
+  if (dot_out && (!dotX || !C->tc_dpart || nrhs > coarse_eo_nt(nrhs)))
     return fail(MGLMA_ERR_INVALID, "coarse_tc_eo: the epilogue dot needs one RHS tile");
   if (par < 0 || par > 1 || d_lo < 0 || d_hi > 8 || d_lo > d_hi)
     return fail(MGLMA_ERR_INVALID, "coarse_tc_eo: bad launch");
   if (Ahop && d_hi > 7) return fail(MGLMA_ERR_INVALID, "coarse_tc_eo: the eight-slot image has no self slot");
-  const int nt = tuned(ctx, TUNE_COARSE_NT, nrhs, C->geo.V1, coarse_tc_default_nt(nrhs));
+  const int nt = coarse_eo_nt(nrhs);
   if (nt == 32)
     return launch_tc_eo<32>(ctx, C, Xhop, Xself, Y, nrhs, mode, par, d_lo, d_hi, Aself, sign, scratch, s, self_image,
                             Ahop, dotX, dot_out, hop_imaged);
@@ -799,14 +799,17 @@ mglma_status coarse_tc_check(mglma_coarse_s* C, cudaStream_t s) {
 
 int coarse_tc_default_nt(int nrhs) { return nrhs <= 8 ? 8 : (nrhs <= 24 ? 16 : 32); }
 
-int coarse_tc_nt(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs) {
-  return tuned(ctx, TUNE_COARSE_NT, nrhs, C->geo.V1, coarse_tc_default_nt(nrhs));
-}
+// RHS per tile of the even-odd launches: all in one tile as far as a tile goes, as
+// the MINRES iteration's three-launch form needs (the width tuned for a lone
+// operator application does not enter: a narrower one turned that form off).
+// Solves to 1e-11, ms, with 8 / 16 / 32 per tile: 12 RHS of 32x16^3 85 / 65 / 70, 17
+// RHS 104 / 97 / 82, 24 RHS of 32^4 555 / 509 / 458, 6 RHS of 8^4 31.4 / 32.2 / 34.5
+int coarse_eo_nt(int nrhs) { return nrhs <= 8 ? 8 : nrhs <= 16 ? 16 : 32; }
 
 mglma_status coarse_x_image_half(mglma_ctx ctx, const mglma_coarse_s* C, const void* X, int nrhs, void* image,
                                  cudaStream_t s) {
   if (nrhs == 0) return MGLMA_OK;
-  const int n2 = C->n2, NT = coarse_tc_nt(ctx, C, nrhs);
+  const int n2 = C->n2, NT = coarse_eo_nt(nrhs);
   const int64_t Vh = C->geo.V1 / 2;
   const size_t groups = (size_t)((nrhs + NT - 1) / NT) * Vh * (n2 / 8) * NT;
   ProfScope ps(ctx, K_COARSE, s);
@@ -825,7 +828,7 @@ mglma_status lanczos_step(mglma_ctx ctx, const mglma_coarse_s* C, double* st, in
     if (v->prec != MGLMA_FP32 || v->n != (size_t)Vh * n2 * 2 || v->nrhs != x.nrhs || n2 % 8)
       return fail(MGLMA_ERR_INVALID, "lanczos_step: FP32 half-lattice fields needed");
   if (x.nrhs == 0) return MGLMA_OK;
-  const int NT = coarse_tc_nt(ctx, C, x.nrhs);
+  const int NT = coarse_eo_nt(x.nrhs);
   const size_t m = (size_t)Vh * (n2 / 2);
   const int nb = (int)std::min<size_t>((m + LZ_T - 1) / LZ_T, 192);
   double2* part = nullptr;

@@ -476,14 +476,14 @@ static mglma_status minres_init(MinresWork& w, const mglma_coarse_s* C, const Ve
 // operator's input image is the previous step's, or the initialisation's) and
 // its update stays pending until the next one or minres_end; w_k sits in
 // direction slot k mod 2.
-static bool minres_unnormalised(const MinresWork& w, const mglma_coarse_s* C, int n, bool eo) {
-  return eo && coarse_schur_dot_ok(w.ctx, C, n, MGLMA_FP32);
+static bool minres_unnormalised(const mglma_coarse_s* C, int n, bool eo) {
+  return eo && coarse_schur_dot_ok(C, n, MGLMA_FP32);
 }
 static mglma_status minres_iter(MinresWork& w, const mglma_coarse_s* C, Vec& x, int n, int k, double tol,
                                 void* scr, size_t scr_bytes, bool eo = false) {
   const int a = k % 3, b = (k + 1) % 3, c = (k + 2) % 3;
   Vec v = w.view(w.Vp, a, n), vo = w.view(w.Vp, c, n), z = w.view(w.Vp, b, n);
-  if (minres_unnormalised(w, C, n, eo)) {
+  if (minres_unnormalised(C, n, eo)) {
     Vec w1 = w.view(w.Wp, k % 2, n), w2 = w.view(w.Wp, (k + 1) % 2, n);  // w_(k-2), w_(k-3)
     MG_CHECK(coarse_schur_apply(w.ctx, C, v.p, z.p, n, MGLMA_FP32, CMODE_Q, scr, scr_bytes, w.s, w.sc.z, true));
     return lanczos_step(w.ctx, C, w.sc.d, w.cap, w.sc.z, w.sc.active, tol, v, vo, z, w1, w2, x, scr, w.s);
@@ -506,7 +506,7 @@ static mglma_status minres_iter(MinresWork& w, const mglma_coarse_s* C, Vec& x, 
 // x after `iters` iterations, iters a multiple of 6: the pending update of the
 // last one (vector slot 2, w_(k-1) in direction slot 0, w_(k-2) in slot 1)
 static mglma_status minres_end(MinresWork& w, const mglma_coarse_s* C, Vec& x, int n, bool eo) {
-  if (!minres_unnormalised(w, C, n, eo)) return MGLMA_OK;
+  if (!minres_unnormalised(C, n, eo)) return MGLMA_OK;
   return minres_flush(w.ctx, w.st(MR_CF), w.cap, w.view(w.Vp, 2, n), w.view(w.Wp, 0, n), w.view(w.Wp, 1, n), x, w.s);
 }
 
@@ -699,7 +699,7 @@ struct CoarseSolver {
       MG_CHECK(minres_init(mw, C, bn, xn));
       // the first Lanczos vector's operator image (the iterations' updates
       // write the later ones)
-      if (coarse_schur_dot_ok(ctx, C, b.nrhs, MGLMA_FP32))
+      if (coarse_schur_dot_ok(C, b.nrhs, MGLMA_FP32))
         MG_CHECK(coarse_x_image_half(ctx, C, mw.view(mw.Vp, 0, b.nrhs).p, b.nrhs, scr, s));
       return MGLMA_OK;
     }

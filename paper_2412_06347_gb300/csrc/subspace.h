@@ -115,7 +115,7 @@ mglma_status coarse_eo_setup(mglma_ctx ctx, mglma_coarse_s* C, cudaStream_t s);
 // operator has its BF16 image, FP64 fields the FP64 operator
 // whether coarse_schur_apply can return <X_r, Y_r> per RHS (dot_out) from
 // its last launch: FP32 on the tensor cores, one RHS tile
-bool coarse_schur_dot_ok(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs, int prec);
+bool coarse_schur_dot_ok(const mglma_coarse_s* C, int nrhs, int prec);
 // x_imaged (with dot_out only): the scratch's first half already holds the
 // image of X_e (coarse_x_image_half / lanczos_step)
 mglma_status coarse_schur_apply(mglma_ctx ctx, const mglma_coarse_s* C, const void* Xe, void* Ye, int nrhs, int prec,
@@ -165,8 +165,8 @@ mglma_status coarse_tc_eo_launch(mglma_ctx ctx, const mglma_coarse_s* C, const f
                                  float sign, void* scratch, cudaStream_t s, const void* self_image = nullptr,
                                  const uint16_t* Ahop = nullptr, const float2* dotX = nullptr,
                                  double2* dot_out = nullptr, bool hop_imaged = false);
-// RHS tile width of the tensor-core coarse launches for nrhs RHS
-int coarse_tc_nt(mglma_ctx ctx, const mglma_coarse_s* C, int nrhs);
+// RHS tile width of the even-odd tensor-core launches for nrhs RHS
+int coarse_eo_nt(int nrhs);
 // the B-operand image (no gamma5hat) of a FP32 half-lattice field X into
 // image (the first half of the even-odd scratch), as the Schur apply's first
 // launch would write it
