@@ -446,9 +446,9 @@ typedef struct {
                            cached blocks -- at most 64, split into equal batches) */
   int coarse_solver;    /* mglma_coarse_solver (MG) */
   int autotune;         /* MG: 1 = the first lockstep batch of each (lattice, RHS
-                           bucket) tunes the stencil and coarse tile shapes
-                           (mglma_autotune) before it runs; 0 = use the table as
-                           it stands (defaults where empty) */
+                           bucket) tunes the stencil (lattices with an odd extent)
+                           and coarse tile shapes (mglma_autotune) before it runs;
+                           0 = use the table as it stands (defaults where empty) */
   int graph;            /* MG: 1 = every FGCR iteration after the first runs as one
                            CUDA graph -- fine stencil, restriction, the coarse
                            MINRES loop as a device-side conditional node that
@@ -559,7 +559,8 @@ mglma_status mglma_serve(mglma_ctx ctx, const mglma_serve_config* cfg, mglma_req
  * events and keeps the fastest in the context, per lattice volume (used by
  * every later call on a lattice of that volume with an RHS count in the same
  * power-of-two bucket):
- *   kernel 0: tile shape of the FP32 stencil, needs g: NR right-hand sides
+ *   kernel 0: tile shape of the FP32 stencil, needs g, timed as a whole
+ *     mglma_dirac_apply (solves use it on lattices with an odd extent): NR right-hand sides
  *     per thread (1, 2, 4) and RW RHS tiles per 128-thread CTA (1, 2, 4;
  *     a CTA then covers 128 / RW sites), coded NR + 16 (RW - 1) (NR = 4 only
  *     with RW = 1); or the staged-tile kernel, 32 sites x NRT RHS per CTA

@@ -4,9 +4,14 @@
 // kernel's RHS per tile (8, 16, 32) are timed with
 // CUDA events on the context stream for a given RHS count, and the fastest
 // is kept per (kernel, RHS bucket, lattice volume) in the context; the table
-// can be saved to and loaded from a text file keyed by GPU name.  The solver
+// can be saved to and loaded from a text file keyed by GPU name.  The stencil is
+// timed as mglma_dirac_apply runs it, between canonical fields: a lone stencil
+// is within 5 % for several shapes, but all except (1,1) need an unpack pass (16
+// RHS of 32x16^3: 348 us at (1,1), 398 to 452 at the others) and take the fused MR
+// steps of a full-lattice solve away.  The solver
 // tunes the shapes of a (lattice, RHS bucket) on its first batch
-// (autotune_for_batch); with MGLMA_TUNE_CACHE naming a file, a context loads
+// (autotune_for_batch; the stencil only on lattices with an odd extent, the
+// others solve on the even-odd one); with MGLMA_TUNE_CACHE naming a file, a context loads
 // that file when created and saves the table after each automatic tuning.
 #include <cstdio>
 #include <cstring>
@@ -55,7 +60,9 @@ static std::string gpu_name(int dev) {
 // Tunes the tile shapes of this (lattice, RHS bucket) unless the context
 // holds them already, and saves the table to the context's cache file.
 mglma_status autotune_for_batch(mglma_ctx ctx, mglma_gauge_s* G, mglma_coarse_s* C, int nrhs) {
-  const bool need_d = !has_tuned(ctx, TUNE_DSLASH32_NR, nrhs, G->g.V);
+  bool even = G->eo_state >= 0;
+  for (int m = 0; m < 4; ++m) even = even && G->g.L[m] % 2 == 0;
+  const bool need_d = !even && !has_tuned(ctx, TUNE_DSLASH32_NR, nrhs, G->g.V);
   const bool need_c = C && C->Aimg && !has_tuned(ctx, TUNE_COARSE_NT, nrhs, C->geo.V1);
   if (!need_d && !need_c) return MGLMA_OK;
   MG_CHECK(mglma_autotune(ctx, need_d ? G : nullptr, need_c ? C : nullptr, nrhs));
@@ -80,13 +87,32 @@ mglma_status mglma_autotune(mglma_ctx ctx, mglma_gauge G, mglma_coarse C, int nr
   const auto key_d = std::make_tuple((int)TUNE_DSLASH32_NR, bucket, G ? G->g.V : (int64_t)0);
   const auto key_c = std::make_tuple((int)TUNE_COARSE_NT, bucket, C ? C->geo.V1 : (int64_t)0);
   if (G && G->ready) {
+    // one canonical field, applied in place (an FP32 application has read all of
+    // its input before it writes), and two FP32 work fields; without room for
+    // them the stencil alone between the work fields
     Spinor a, b;
     FreeList fl(ctx, s);
-    st = alloc_spinor(ctx, a, MGLMA_FP32, nrhs, G->g.V, s);
-    if (st == MGLMA_OK) st = alloc_spinor(ctx, b, MGLMA_FP32, nrhs, G->g.V, s);
-    fl.add(a.p);
-    fl.add(b.p);
-    if (st == MGLMA_OK) MG_CUDA(cudaMemsetAsync(a.p, 0, a.bytes(), s));
+    const size_t field = (size_t)nrhs * G->g.V * 24;
+    void *work = nullptr, *canon = nullptr;
+    a.prec = b.prec = MGLMA_FP32;
+    a.nrhs = b.nrhs = nrhs;
+    a.V = b.V = G->g.V;
+    const size_t off = (a.bytes() + 255) / 256 * 256;
+    st = dalloc(ctx, &work, off + b.bytes(), s);
+    fl.add(work);
+    if (st == MGLMA_OK) {
+      a.p = work;
+      b.p = (char*)work + off;
+      MG_CUDA(cudaMemsetAsync(work, 0, off + b.bytes(), s));
+      if (dalloc(ctx, &canon, field * sizeof(double), s) == MGLMA_OK)
+        MG_CUDA(cudaMemsetAsync(canon, 0, field * sizeof(double), s));
+      fl.add(canon);
+    }
+    auto apply = [&] {
+      double* c = (double*)canon;
+      return c ? dirac_canonical(ctx, G, MGLMA_OP_D, nrhs, c, c, MGLMA_FP32, work, s)
+               : dslash(ctx, G, a, b, false, false, s);
+    };
     double best = 1e30;
     int choice = 1;
     // {NR, RW} of the one-site-per-thread kernel; {0, NRT} the staged-tile kernel
@@ -98,7 +124,7 @@ mglma_status mglma_autotune(mglma_ctx ctx, mglma_gauge G, mglma_coarse C, int nr
       const int code = sh[0] ? dslash32_tile_code(sh[0], sh[1]) : 64 + sh[1];
       ctx->tune[key_d] = {code, 0.0};
       double ms = 0;
-      st = time_ms(ctx, s, 5, [&] { return dslash(ctx, G, a, b, false, false, s); }, &ms);
+      st = time_ms(ctx, s, 5, apply, &ms);
       if (st == MGLMA_OK && ms < best) {
         best = ms;
         choice = code;
