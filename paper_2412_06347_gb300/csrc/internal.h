@@ -356,8 +356,8 @@ mglma_status schur_dot(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const
 mglma_status schur_mr_step(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& t, Spinor& tn,
                            const Spinor& sk, Spinor& sn, const float2* alpha, float2* alpha_n, double* part,
                            cudaStream_t s);
-mglma_status mr_iterate(mglma_ctx, Spinor& z, const void* s0, size_t sstride_bytes, int ns, const float2* alpha,
-                        cudaStream_t s);
+mglma_status mr_iterate(mglma_ctx, Spinor& z, const void* s0, int sprec, size_t sstride_bytes, int ns,
+                        const float2* alpha, cudaStream_t s);
 mglma_status schur_gcr(mglma_ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out, int k,
                        const void* W0, size_t wslot_reals, const void* r, double* part, double* nw, double2* num,
                        double2* dots, cudaStream_t s);

@@ -867,7 +867,7 @@ struct TwoLevel {
   Scalars sc;
   CoarseSolver cs;
   bool ready = false;
-  bool fused = false;      // fused MR steps on BF16 s, t
+  bool fused = false;      // BF16 s, t; on the full lattice fused MR steps
   bool tc_r0 = false;      // R0 on the tensor cores (BF16 operands; the coarse solve is BF16 already)
   bool tc_t0 = false;      // T0 on the tensor cores (BF16 operands)
   bool half_r0 = false, half_t0 = false;  // ... on half fields
@@ -897,8 +897,10 @@ struct TwoLevel {
     MG_CHECK(dalloc(ctx, &e1.p, e1.bytes(), s));
     // the smoother's s and t: BF16 on the fused path (the flexible outer
     // solve takes the rounded preconditioner; measured: same FGCR and coarse
-    // iteration counts as FP32 at 64x32^3), FP32 otherwise
-    fused = eo || (p->nu > 1 && dslash_mr_fused(ctx, G, n));
+    // iteration counts as FP32 at 64x32^3), FP32 otherwise: for one step on D, and
+    // where a staged stencil tile was set, which has no fused steps; the even-odd
+    // form, which has both, follows the same rule
+    fused = p->nu > 1 && dslash_mr_fused(ctx, G, n);
     // in even-odd form on the even sites where the half blocks fit, else on a
     // full field
     half_r0 = eo && n >= 8 && restrict_tc_supported(C->sub, true);
@@ -912,7 +914,7 @@ struct TwoLevel {
     tv = tv2 = sv;
     MG_CHECK(dalloc(ctx, &sv.p, sv.bytes() * (eo ? std::min(kGroup, std::max(1, schur_steps(p->nu))) : 1), s));
     MG_CHECK(dalloc(ctx, &tv.p, tv.bytes(), s));
-    if (fused) MG_CHECK(dalloc(ctx, &tv2.p, tv2.bytes(), s));
+    if (fused || eo) MG_CHECK(dalloc(ctx, &tv2.p, tv2.bytes(), s));
     if (eo) {
       wo = full = r;
       wo.nrhs = full.nrhs = n;
@@ -1054,7 +1056,7 @@ struct TwoLevel {
       if (k % kGroup == 0) {
         // the next slot reuses the group's first: its sum goes into z first,
         // its last alpha moves out of the way of the new group
-        MG_CHECK(mr_iterate(ctx, z, sv.p, stride, kGroup, al, s));
+        MG_CHECK(mr_iterate(ctx, z, sv.p, sv.prec, stride, kGroup, al, s));
         MG_CUDA(cudaMemcpyAsync(al + (size_t)kGroup * n, alpha(k - 1), sizeof(float2) * n, cudaMemcpyDeviceToDevice, s));
         MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, al + (size_t)kGroup * n, alpha(k), part, s));
       } else {
@@ -1062,7 +1064,7 @@ struct TwoLevel {
       }
       std::swap(tc, tn);
     }
-    return mr_iterate(ctx, z, sv.p, stride, (steps - 1) % kGroup + 1, al, s);
+    return mr_iterate(ctx, z, sv.p, sv.prec, stride, (steps - 1) % kGroup + 1, al, s);
   }
 };
 

@@ -15,7 +15,7 @@
 //   odd pass   w_o = A_oo^-1 H_oe x_e
 //   even pass  y_e = A_ee x_e - H_eo w_o, with what follows it (residual,
 //              dots, a whole MR step) in the epilogue.
-// w is FP32; x is FP32, or BF16 for the smoother's fields.
+// w is FP32; x is FP32, or BF16 for the smoother's fields (FP32 too when asked for).
 //
 // What bounds it: nothing alone.  ncu on 32^4, 16 RHS (odd pass, BF16 in): FMA
 // pipe 50 %, issue slots 49 %, L1 51 %, DRAM 37 %, long-scoreboard stalls 4.5
@@ -423,10 +423,10 @@ __global__ void __launch_bounds__(SCHUR_T, schur_ctas<-1>())
 enum {
   EV_APPLY,  // out = S x                                            (FP32)
   EV_PREP,  // out = b - H_eo w                                     (FP32)
-  EV_RES,   // out = b - S x                                        (FP32 b; out BF16)
-  EV_DOT,   // out = S x, partials of |out|^2 and <out, x>          (BF16 x, out)
+  EV_RES,   // out = b - S x                                        (FP32 b; out SM)
+  EV_DOT,   // out = S x, partials of |out|^2 and <out, x>          (SM x, out)
   EV_MR,    // one MR step: with u = S x (x = t_k): out = t_k - a u, sn = s - a t_k,
-            // partials of |out|^2 and <out, sn>                     (BF16)
+            // partials of |out|^2 and <out, sn>                     (SM)
   EV_GCR    // out = S x with the FGCR dots                         (FP32)
 };
 struct EvArgs {
@@ -456,14 +456,15 @@ __device__ __forceinline__ void warp_partials(float* v, double* acc) {
     for (int e = 0; e < NV; ++e) acc[e] += (double)v[e];
 }
 
-template <int EV>
+// SM: storage of the smoother's fields, SpinBf16 or float
+template <int EV, typename SM = SpinBf16>
 __global__ void __launch_bounds__(SCHUR_T, schur_ctas<EV>())
     schur_even_kernel(const void* __restrict__ w, const void* __restrict__ x, void* __restrict__ out, EoLinks U,
                       const char* __restrict__ C, EoGeo g, int nrhs, int nsub, EvArgs a) {
   constexpr bool RED = EV == EV_DOT || EV == EV_MR || EV == EV_GCR;
-  constexpr bool BFX = EV == EV_DOT || EV == EV_MR;
   constexpr int NV = EV == EV_GCR ? 6 : 3;
-  using SX = typename std::conditional<BFX, SpinBf16, float>::type;
+  constexpr bool BF = std::is_same<SM, SpinBf16>::value;
+  using SX = typename std::conditional<EV == EV_DOT || EV == EV_MR, SM, float>::type;
   const EoTile t(g, nrhs);
   const int r = t.r;
   __shared__ double sum[NV];  // thread 0's
@@ -507,42 +508,63 @@ __global__ void __launch_bounds__(SCHUR_T, schur_ctas<EV>())
         q.load(rhs_of<float>(a.b, g, r), g.Vh, u);
 #pragma unroll
         for (int j = 0; j < 12; ++j) acc[j] = adds<-1>(q.get(j), acc[j]);
-        Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
+        Sp<SM>::store(rhs_of<SM>(out, g, r), g.Vh, u, acc);
       } else if (EV == EV_DOT) {
-        Sp<SpinBf16> p;
-        p.load(rhs_of<SpinBf16>(x, g, r), g.Vh, u);
+        Sp<SM> p;
+        p.load(rhs_of<SM>(x, g, r), g.Vh, u);
 #pragma unroll
         for (int j = 0; j < 12; ++j) {
-          const float2 q = unpack2(pack2(acc[j])), y = p.get(j);  // the dots see the values as stored
+          const float2 q = BF ? unpack2(pack2(acc[j])) : acc[j], y = p.get(j);  // the dots see the values as stored
           acc[j] = q;
           v[0] += q.x * q.x + q.y * q.y;
           v[1] += q.x * y.x + q.y * y.y;
           v[2] += q.x * y.y - q.y * y.x;
         }
-        Sp<SpinBf16>::store(rhs_of<SpinBf16>(out, g, r), g.Vh, u, acc);
+        Sp<SM>::store(rhs_of<SM>(out, g, r), g.Vh, u, acc);
       } else if (EV == EV_MR) {
         const float2 al = a.alpha[r];
         // complex -a v = nr (re, im) + ni (im, re) with ni = (Im a, -Im a)
         const float2 nr = dup(-al.x), ni = make_float2(al.y, -al.y);
-        const char *tp = rhs_of<SpinBf16>(x, g, r), *sp = rhs_of<SpinBf16>(a.s, g, r);
-        char *op = rhs_of<SpinBf16>(out, g, r), *np = rhs_of<SpinBf16>(a.sn, g, r);
+        const char *tp = rhs_of<SM>(x, g, r), *sp = rhs_of<SM>(a.s, g, r);
+        char *op = rhs_of<SM>(out, g, r), *np = rhs_of<SM>(a.sn, g, r);
+        if constexpr (BF) {
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const uint4 tv = ldg_row<uint4>(tp, g.Vh, j, u), sv = ldg_row<uint4>(sp, g.Vh, j, u);
-          const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w}, sw[4] = {sv.x, sv.y, sv.z, sv.w};
-          uint32_t to[4], so[4];
+          for (int j = 0; j < 3; ++j) {
+            const uint4 tv = ldg_row<uint4>(tp, g.Vh, j, u), sv = ldg_row<uint4>(sp, g.Vh, j, u);
+            const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w}, sw[4] = {sv.x, sv.y, sv.z, sv.w};
+            uint32_t to[4], so[4];
 #pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            const float2 tk = unpack2(tw[h]), sk = unpack2(sw[h]), q = acc[4 * j + h];
-            to[h] = pack2(fma2(ni, make_float2(q.y, q.x), fma2(nr, q, tk)));
-            so[h] = pack2(fma2(ni, make_float2(tk.y, tk.x), fma2(nr, tk, sk)));
-            const float2 tn = unpack2(to[h]), sn = unpack2(so[h]);
-            v[0] += tn.x * tn.x + tn.y * tn.y;
-            v[1] += tn.x * sn.x + tn.y * sn.y;
-            v[2] += tn.x * sn.y - tn.y * sn.x;
+            for (int h = 0; h < 4; ++h) {
+              const float2 tk = unpack2(tw[h]), sk = unpack2(sw[h]), q = acc[4 * j + h];
+              to[h] = pack2(fma2(ni, make_float2(q.y, q.x), fma2(nr, q, tk)));
+              so[h] = pack2(fma2(ni, make_float2(tk.y, tk.x), fma2(nr, tk, sk)));
+              const float2 tn = unpack2(to[h]), sn = unpack2(so[h]);
+              v[0] += tn.x * tn.x + tn.y * tn.y;
+              v[1] += tn.x * sn.x + tn.y * sn.y;
+              v[2] += tn.x * sn.y - tn.y * sn.x;
+            }
+            row<uint4>(op, g.Vh, j, u) = make_uint4(to[0], to[1], to[2], to[3]);
+            row<uint4>(np, g.Vh, j, u) = make_uint4(so[0], so[1], so[2], so[3]);
           }
-          row<uint4>(op, g.Vh, j, u) = make_uint4(to[0], to[1], to[2], to[3]);
-          row<uint4>(np, g.Vh, j, u) = make_uint4(so[0], so[1], so[2], so[3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            const float4 tv = ldg_row<float4>(tp, g.Vh, j, u), sv = ldg_row<float4>(sp, g.Vh, j, u);
+            const float2 tk[2] = {make_float2(tv.x, tv.y), make_float2(tv.z, tv.w)};
+            const float2 sk[2] = {make_float2(sv.x, sv.y), make_float2(sv.z, sv.w)};
+            float2 tn[2], sn[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 q = acc[2 * j + h];
+              tn[h] = fma2(ni, make_float2(q.y, q.x), fma2(nr, q, tk[h]));
+              sn[h] = fma2(ni, make_float2(tk[h].y, tk[h].x), fma2(nr, tk[h], sk[h]));
+              v[0] += tn[h].x * tn[h].x + tn[h].y * tn[h].y;
+              v[1] += tn[h].x * sn[h].x + tn[h].y * sn[h].y;
+              v[2] += tn[h].x * sn[h].y - tn[h].y * sn[h].x;
+            }
+            row<float4>(op, g.Vh, j, u) = make_float4(tn[0].x, tn[0].y, tn[1].x, tn[1].y);
+            row<float4>(np, g.Vh, j, u) = make_float4(sn[0].x, sn[0].y, sn[1].x, sn[1].y);
+          }
         }
       } else {
         Sp<float>::store(rhs_of<float>(out, g, r), g.Vh, u, acc);
@@ -619,32 +641,43 @@ __global__ void __launch_bounds__(512) mr_finish_kernel(const double* __restrict
   }
 }
 
-// z += sum_{k<ns} alpha_k s_k (s_k at s + k sstride uint4, alpha_k[rhs] at alpha
-// + k nrhs): the smoothing steps' iterate, formed once per group of steps, so a
-// step moves 288 B per site and RHS instead of 480.  One thread per site and
-// group of four components
-template <int NS>
+// z += sum_{k<ns} alpha_k s_k (s_k at s + k sstride 16-byte pieces, alpha_k[rhs] at
+// alpha + k nrhs): the smoothing steps' iterate, formed once per group of steps, so
+// a step moves 288 B per site and RHS instead of 480 (BF16 s_k).  One thread per
+// site and group of four components
+template <int NS, typename SM>
 __global__ void __launch_bounds__(256) mr_iterate_kernel(float4* __restrict__ z, const uint4* __restrict__ s,
                                                          size_t sstride, const float2* __restrict__ alpha, int nrhs,
                                                          uint32_t Vh) {
+  constexpr bool BF = std::is_same<SM, SpinBf16>::value;
+  constexpr int PIECES = BF ? 1 : 2;  // per group of four components
   const int r = blockIdx.y;
   const uint32_t j = blockIdx.z, u = blockIdx.x * 256 + threadIdx.x;
   if (u >= Vh) return;
-  const uint4* sp = s + ((size_t)r * 3 + j) * Vh + u;
+  const uint4* sp = s + ((size_t)r * 3 + j) * PIECES * Vh + u;
   float4* z0 = z + ((size_t)r * 6 + 2 * j) * Vh + u;
-  uint4 sv[NS];
+  uint4 sv[NS][PIECES];
 #pragma unroll
-  for (int k = 0; k < NS; ++k) sv[k] = __ldg(sp + k * sstride);
+  for (int k = 0; k < NS; ++k)
+#pragma unroll
+    for (int p = 0; p < PIECES; ++p) sv[k][p] = __ldg(sp + k * sstride + (size_t)p * Vh);
   const float4 a = z0[0], c = z0[Vh];
   float2 q[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(c.x, c.y), make_float2(c.z, c.w)};
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const float2 al = alpha[(size_t)k * nrhs + r];
     const float2 ar = dup(al.x), ai = make_float2(-al.y, al.y);
-    const uint32_t w[4] = {sv[k].x, sv[k].y, sv[k].z, sv[k].w};
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      const float2 v = unpack2(w[h]);
+      float2 v;
+      if constexpr (BF) {
+        const uint32_t w[4] = {sv[k][0].x, sv[k][0].y, sv[k][0].z, sv[k][0].w};
+        v = unpack2(w[h]);
+      } else {
+        const uint4 w = sv[k][h / 2];
+        v = h % 2 ? make_float2(__uint_as_float(w.z), __uint_as_float(w.w))
+                  : make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+      }
       q[h] = fma2(ai, make_float2(v.y, v.x), fma2(ar, v, q[h]));
     }
   }
@@ -901,10 +934,10 @@ mglma_status schur_odd_solution(mglma_ctx ctx, const mglma_gauge_s* G, const Spi
   return MGLMA_OK;
 }
 
-template <int EV>
+template <int EV, typename SM = SpinBf16>
 static void launch_even(const mglma_gauge_s* G, const Spinor& w, const void* x, void* out, const EvArgs& a,
                         cudaStream_t s) {
-  schur_even_kernel<EV><<<schur_blocks(G) * (unsigned)w.nrhs, SCHUR_T, 0, s>>>(
+  schur_even_kernel<EV, SM><<<schur_blocks(G) * (unsigned)w.nrhs, SCHUR_T, 0, s>>>(
       w.p, x, out, eo_links(G), G->Ceo, launch_geo(G, w.nrhs), w.nrhs, (int)eo_nsub((uint32_t)(G->g.V / 2)), a);
 }
 
@@ -936,8 +969,12 @@ mglma_status schur_resid(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& w,
   if (out.nrhs == 0) return MGLMA_OK;
   EvArgs a;
   a.b = b.p;
-  ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, out.nrhs, 336.0), schur_flops(G, out.nrhs));
-  launch_even<EV_RES>(G, w, x.p, out.p, a, s);
+  const bool bf = out.prec == MGLMA_BF16;
+  ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, out.nrhs, bf ? 336.0 : 384.0), schur_flops(G, out.nrhs));
+  if (bf)
+    launch_even<EV_RES>(G, w, x.p, out.p, a, s);
+  else
+    launch_even<EV_RES, float>(G, w, x.p, out.p, a, s);
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
 }
@@ -956,12 +993,17 @@ static mglma_status mr_finish(mglma_ctx ctx, const mglma_gauge_s* G, const doubl
 mglma_status schur_dot(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out,
                        double* part, float2* alpha, cudaStream_t s) {
   MG_CHECK(eo_shape(G, {&out, &w, &x}, "schur_dot"));
+  if (x.prec != out.prec) return fail(MGLMA_ERR_INVALID, "schur_dot: fields of one precision needed");
   if (out.nrhs == 0) return MGLMA_OK;
   EvArgs a;
   a.part = part;
   {
-    ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, out.nrhs, 192.0), schur_flops(G, out.nrhs));
-    launch_even<EV_DOT>(G, w, x.p, out.p, a, s);
+    const bool bf = out.prec == MGLMA_BF16;
+    ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, out.nrhs, bf ? 192.0 : 288.0), schur_flops(G, out.nrhs));
+    if (bf)
+      launch_even<EV_DOT>(G, w, x.p, out.p, a, s);
+    else
+      launch_even<EV_DOT, float>(G, w, x.p, out.p, a, s);
   }
   MG_LAUNCH_CHECK();
   return mr_finish(ctx, G, part, out.nrhs, alpha, s);
@@ -971,6 +1013,8 @@ mglma_status schur_mr_step(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& 
                            const Spinor& sk, Spinor& sn, const float2* alpha, float2* alpha_n, double* part,
                            cudaStream_t s) {
   MG_CHECK(eo_shape(G, {&tn, &w, &t, &sk, &sn}, "schur_mr_step"));
+  if (t.prec != tn.prec || sk.prec != tn.prec || sn.prec != tn.prec)
+    return fail(MGLMA_ERR_INVALID, "schur_mr_step: fields of one precision needed");
   if (tn.nrhs == 0) return MGLMA_OK;
   EvArgs a;
   a.s = sk.p;
@@ -978,30 +1022,40 @@ mglma_status schur_mr_step(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& 
   a.alpha = alpha;
   a.part = part;
   {
-    ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, tn.nrhs, 288.0), schur_flops(G, tn.nrhs));
-    launch_even<EV_MR>(G, w, t.p, tn.p, a, s);
+    const bool bf = tn.prec == MGLMA_BF16;
+    ProfScope ps(ctx, K_DSLASH32, s, schur_bytes(G, tn.nrhs, bf ? 288.0 : 480.0), schur_flops(G, tn.nrhs));
+    if (bf)
+      launch_even<EV_MR>(G, w, t.p, tn.p, a, s);
+    else
+      launch_even<EV_MR, float>(G, w, t.p, tn.p, a, s);
   }
   MG_LAUNCH_CHECK();
   return mr_finish(ctx, G, part, tn.nrhs, alpha_n, s);
 }
 
-mglma_status mr_iterate(mglma_ctx ctx, Spinor& z, const void* s0, size_t sstride_bytes, int ns, const float2* alpha,
-                        cudaStream_t s) {
-  if (z.nrhs == 0) return MGLMA_OK;
+template <typename SM>
+static mglma_status launch_iterate(Spinor& z, const uint4* sp, size_t st, int ns, const float2* alpha,
+                                   cudaStream_t s) {
   const uint32_t Vh = (uint32_t)z.V;
-  ProfScope ps(ctx, K_BLAS, s, (192.0 + 48.0 * ns) * (double)z.V * z.nrhs);
   const dim3 g((Vh + 255) / 256, z.nrhs, 3);
-  const uint4* sp = (const uint4*)s0;
-  const size_t st = sstride_bytes / 16;
   switch (ns) {
-    case 1: mr_iterate_kernel<1><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
-    case 2: mr_iterate_kernel<2><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
-    case 3: mr_iterate_kernel<3><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
-    case 4: mr_iterate_kernel<4><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
+    case 1: mr_iterate_kernel<1, SM><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
+    case 2: mr_iterate_kernel<2, SM><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
+    case 3: mr_iterate_kernel<3, SM><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
+    case 4: mr_iterate_kernel<4, SM><<<g, 256, 0, s>>>((float4*)z.p, sp, st, alpha, z.nrhs, Vh); break;
     default: return fail(MGLMA_ERR_INVALID, "mr_iterate: 1 to 4 steps");
   }
   MG_LAUNCH_CHECK();
   return MGLMA_OK;
+}
+
+mglma_status mr_iterate(mglma_ctx ctx, Spinor& z, const void* s0, int sprec, size_t sstride_bytes, int ns,
+                        const float2* alpha, cudaStream_t s) {
+  if (z.nrhs == 0) return MGLMA_OK;
+  const bool bf = sprec == MGLMA_BF16;
+  ProfScope ps(ctx, K_BLAS, s, (192.0 + (bf ? 48.0 : 96.0) * ns) * (double)z.V * z.nrhs);
+  if (bf) return launch_iterate<SpinBf16>(z, (const uint4*)s0, sstride_bytes / 16, ns, alpha, s);
+  return launch_iterate<float>(z, (const uint4*)s0, sstride_bytes / 16, ns, alpha, s);
 }
 
 mglma_status schur_gcr(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& w, const Spinor& x, Spinor& out, int k,

@@ -7,8 +7,7 @@
 // can be saved to and loaded from a text file keyed by GPU name.  The stencil is
 // timed as mglma_dirac_apply runs it, between canonical fields: a lone stencil
 // is within 5 % for several shapes, but all except (1,1) need an unpack pass (16
-// RHS of 32x16^3: 348 us at (1,1), 398 to 452 at the others) and take the fused MR
-// steps of a full-lattice solve away.  The solver
+// RHS of 32x16^3: 348 us at (1,1), 398 to 452 at the others).  The solver
 // tunes the shapes of a (lattice, RHS bucket) on its first batch
 // (autotune_for_batch; the stencil only on lattices with an odd extent, the
 // others solve on the even-odd one); with MGLMA_TUNE_CACHE naming a file, a context loads
