@@ -145,7 +145,8 @@ struct mglma_gauge_s {
   // not tried
   char *Ueo = nullptr, *Ceo = nullptr, *Ieo = nullptr;
   int eo_state = 0;
-  std::mutex eo_mu;
+  int eo_users = 0;  // solves that hold them (EoUse)
+  std::mutex eo_mu;  // guards the copies above and the double-float ones
   int slabs_loaded = 0;   // time slices received
   std::vector<char> slab_seen;
   bool ready = false;
@@ -312,6 +313,8 @@ mglma_status dslash_mr_step(mglma_ctx, const mglma_gauge_s* G, const Spinor& t, 
 // r -= scale[rhs] D e per RHS: e FP32, r FP64, D applied in double-float
 // arithmetic (about 2^-47 relative to the terms) on the FP64 links and clover
 // split once into double-float words (kept on the gauge handle)
+// (gauge_df_ready forms the copies it needs, on first use; waits for them)
+mglma_status gauge_df_ready(mglma_gauge_s* G, cudaStream_t s);
 mglma_status dslash_resid_df(mglma_ctx ctx, const mglma_gauge_s* G, const Spinor& e, Spinor& r, const double* scale,
                              cudaStream_t s);
 mglma_status dslash_resid(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, const Spinor& b, Spinor& out,
@@ -327,6 +330,22 @@ size_t dslash_dot_part_doubles(int64_t V, int nrhs);
 // Forms the parity-split copies on first use; *usable false (and MGLMA_OK)
 // when an extent is odd, a clover block has no good inverse or memory is short.
 mglma_status fine_eo_ready(mglma_ctx, mglma_gauge_s* G, bool* usable, cudaStream_t s);
+// A solve's hold on the copies: they stay while one exists.  drop gives the hold
+// up and frees the copies unless another solve holds them (a solve that ran out
+// of memory makes room that way and takes the full-lattice system).
+struct EoUse {
+  mglma_gauge_s* G = nullptr;
+  bool usable = false;
+  EoUse() = default;
+  EoUse(const EoUse&) = delete;
+  EoUse& operator=(const EoUse&) = delete;
+  ~EoUse() { release(false); }
+  mglma_status acquire(mglma_ctx, const mglma_gauge_s* g, cudaStream_t s);
+  void drop() { release(true); }
+
+ private:
+  void release(bool free);
+};
 // odd pass: w = A_oo^-1 H_oe in (in FP32 or BF16, w FP32)
 mglma_status schur_odd(mglma_ctx, const mglma_gauge_s* G, const Spinor& in, Spinor& w, cudaStream_t s);
 // x_o = A_oo^-1 (b_o - H_oe x_e); without xe: A_oo^-1 b_o (FP32)

@@ -1068,6 +1068,16 @@ struct TwoLevel {
   }
 };
 
+// device bytes per lattice site and RHS of the FP32 system: source, solution (and
+// the odd source), FGCR(m), and the preconditioner's fine fields with the full field
+// that transfers without a half form go through
+static size_t fp32_site_bytes(bool eo, int m, int nu, bool bf) {
+  const size_t f = eo ? 48 : 96, sm = bf && nu > 1 ? f / 2 : f;  // a field, a smoother field
+  const int held = eo ? std::min(TwoLevel::kGroup, std::max(1, schur_steps(nu))) : 1;
+  return (eo ? 3 : 2) * f + (2 * (size_t)m + 1) * f + (held + (eo || (bf && nu > 1) ? 2 : 1)) * sm +
+         (eo ? f + 2 * f : 0);
+}
+
 // Inner-tolerance factor for a RHS at FP64 relative residual `rel`: when
 // this cycle can reach the target (inner_tol * rel < 10 tol), the inner solve
 // aims at 0.3 tol / rel instead of inner_tol -- tighter when two cycles of
@@ -1079,17 +1089,16 @@ static double final_cycle_scale(const MgParams& p, double rel) {
 }
 
 // x (FP64, zero on entry) = D^-1 b to p.tol in the FP64 residual.
-mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_s* C, const Spinor& b, Spinor& x,
-                      const MgParams& p, std::vector<RhsStat>& out, cudaStream_t s) {
+// even_odd: the FP32 solve runs on the Schur system of the even sites (schur.cu);
+// r32 / e32 are then its source and solution (half fields), ro the odd part of r /
+// |r|, eo the odd part of the correction.  Its copies must exist.
+static mglma_status mg_solve_form(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_s* C, const Spinor& b,
+                                  Spinor& x, const MgParams& p, std::vector<RhsStat>& out, cudaStream_t s,
+                                  bool even_odd) {
   const int n = b.nrhs;
   const int64_t V = b.V;
   out.assign(n, RhsStat());
   FreeList fl(ctx, s);
-  // With every extent even the FP32 solve runs on the Schur system of the
-  // even sites (schur.cu): r32 / e32 are then its source and solution (half
-  // fields), ro the odd part of r / |r|, eo the odd part of the correction
-  bool even_odd = false;
-  MG_CHECK(fine_eo_ready(ctx, const_cast<mglma_gauge_s*>(G), &even_odd, s));
   const int64_t Vs = even_odd ? V / 2 : V;  // sites of the FP32 system
   Spinor r, r32, e32, re, ro, eo, ef;
   MG_CHECK(alloc_spinor(ctx, r, MGLMA_FP64, n, V, s));
@@ -1215,6 +1224,30 @@ mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_
   for (int i = 0; i < n; ++i) out[i].coarse_iterations = K.coarse_iters;
   if (K.tc_r0 || K.tc_t0) MG_CHECK(restrict_tc_check(C->sub, s));
   return coarse_tc_check(const_cast<mglma_coarse_s*>(C), s);
+}
+
+size_t mg_site_bytes(bool even_odd, int gcr_m, int nu, bool bf16_smoother) {
+  // FP64 b, x, r; the FP32 system and its preconditioner; e on both parities and
+  // whole, the residual's even part
+  const size_t fp64 = 3 * 192, sys = fp32_site_bytes(even_odd, gcr_m, nu, bf16_smoother);
+  return fp64 + sys + (even_odd ? 2 * 48 + 96 : 0);
+}
+
+mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_s* C, const Spinor& b, Spinor& x,
+                      const MgParams& p, std::vector<RhsStat>& out, cudaStream_t s) {
+  // what either form needs first, then the even-odd copies (every extent even) if
+  // there is room; when the even-odd form finds none for its fields, the copies go
+  // and the full-lattice form has the whole room
+  MG_CHECK(gauge_df_ready(const_cast<mglma_gauge_s*>(G), s));
+  EoUse copies;
+  MG_CHECK(copies.acquire(ctx, G, s));
+  const mglma_status st = mg_solve_form(ctx, G, C, b, x, p, out, s, copies.usable);
+  if (st != MGLMA_ERR_OOM || !copies.usable) return st;
+  MG_CUDA(cudaStreamSynchronize(s));
+  copies.drop();
+  MG_CUDA(cudaMemPoolTrimTo(ctx->pool, 0));
+  MG_CUDA(cudaMemsetAsync(x.p, 0, x.bytes(), s));
+  return mg_solve_form(ctx, G, C, b, x, p, out, s, false);
 }
 
 // rn = |r|, rinv = 1 / |r| for the RHS still iterating, 0 for the others
@@ -1437,13 +1470,17 @@ struct Engine {
   FreeList* fl = nullptr;
   static constexpr int kInnerCap = 400;
 
+  EoUse copies;  // of the gauge field's even-odd stencil
+
   // device bytes one slot needs (FP64 b, x, r -- r also holds D x while the
-  // residual is formed; FP32 r, e, FGCR directions and images, preconditioner
-  // scratch)
-  static size_t slot_bytes(int64_t V, int m) { return (size_t)V * (3 * 192 + (size_t)(6 + 2 * m) * 96); }
-  // one canonical spinor that host requests pass through, allocated on the
-  // first host request (device requests need none)
-  static size_t fixed_bytes(int64_t) { return 0; }
+  // residual is formed; the FP32 system and its preconditioner; the coarse fields
+  // are a few per cent of that)
+  static size_t slot_bytes(int64_t V, const MgParams& p, bool eo, bool bf) {
+    return (size_t)V * (3 * 192 + fp32_site_bytes(eo, p.gcr_m, p.nu, bf));
+  }
+  // and the lattice as such, besides the copies: one slot's temporaries.  (The
+  // canonical spinor that host requests pass through comes with the first one.)
+  static size_t fixed_bytes(int64_t V, bool eo) { return eo ? (size_t)V * (2 * 48 + 96) : 0; }
   mglma_status ensure_stage() {
     if (stage) return MGLMA_OK;
     MG_CHECK(dalloc(ctx, (void**)&stage, (size_t)V * 24 * sizeof(double), s));
@@ -1453,6 +1490,7 @@ struct Engine {
 
   ~Engine() { delete fl; }
 
+  // the even-odd copies, when they can be formed, stay this engine's
   mglma_status setup(mglma_ctx c, cudaStream_t st, const mglma_gauge_s* g, const mglma_coarse_s* co,
                      const MgParams& prm, int capacity) {
     ctx = c;
@@ -1462,12 +1500,12 @@ struct Engine {
     p = prm;
     cap = capacity;
     V = g->g.V;
+    even_odd = copies.usable;
     fl = new FreeList(ctx, s);
     for (Spinor* f : {&b64, &x64, &r64}) {
       MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP64, cap, V, s));
       fl->add(f->p);
     }
-    MG_CHECK(fine_eo_ready(ctx, const_cast<mglma_gauge_s*>(G), &even_odd, s));
     Vs = even_odd ? V / 2 : V;
     for (Spinor* f : {&r32, &e32}) {
       MG_CHECK(alloc_spinor(ctx, *f, MGLMA_FP32, cap, Vs, s));
@@ -1494,6 +1532,7 @@ struct Engine {
     K.p = &p;
     K.cap = cap;
     K.eo = even_odd;
+    MG_CHECK(K.setup(as_vec(r32)));
     MG_CHECK(fill_int(gw.sc.active, 0, cap, s));
     slots.assign(cap, Slot());
     return MGLMA_OK;
@@ -1668,13 +1707,38 @@ extern "C" mglma_status mglma_serve(mglma_ctx ctx, const mglma_serve_config* cfg
     const mglma_serve_lattice& L = cfg->lattices[l];
     if (!L.gauge || !L.coarse || L.coarse->sub->gauge != L.gauge)
       return fail(MGLMA_ERR_INVALID, "serve: lattice entries need a gauge field and its coarse operator");
-    const size_t per = Engine::slot_bytes(L.gauge->g.V, mp.gcr_m);
-    const double share =
-        cfg->hbm_fraction * (double)fr * ((double)L.gauge->g.V / vsum) - (double)Engine::fixed_bytes(L.gauge->g.V);
-    const int cap = share > 0 ? (int)std::min<size_t>((size_t)cfg->max_slots, (size_t)(share / per)) : 0;
-    if (cap < 1) return fail(MGLMA_ERR_OOM, "serve: not enough free HBM for one slot of lattice " + std::to_string(l));
-    eng[l].reset(new Engine());
-    MG_CHECK(eng[l]->setup(ctx, s, L.gauge, L.coarse, mp, cap));
+    // the even-odd form if its copies and one slot fit into the lattice's share,
+    // else the full-lattice form
+    const int64_t V = L.gauge->g.V;
+    const bool bf = dslash_mr_fused(ctx, L.gauge, cfg->max_slots);
+    mglma_status got = MGLMA_ERR_OOM;
+    size_t per = 0;
+    int cap = 0;
+    for (int form = 1; form >= 0 && got == MGLMA_ERR_OOM; --form) {
+      eng[l].reset(new Engine());
+      double share = cfg->hbm_fraction * (double)fr * ((double)V / vsum);
+      if (form) {
+        const size_t before = device_room(ctx, s);
+        MG_CHECK(eng[l]->copies.acquire(ctx, L.gauge, s));
+        if (!eng[l]->copies.usable) continue;
+        const size_t after = device_room(ctx, s);
+        share -= before > after ? (double)(before - after) : 0.0;
+      }
+      per = Engine::slot_bytes(V, mp, form, bf);
+      share -= (double)Engine::fixed_bytes(V, form);
+      cap = share > 0 ? (int)std::min<size_t>((size_t)cfg->max_slots, (size_t)(share / per)) : 0;
+      if (cap >= 1) got = eng[l]->setup(ctx, s, L.gauge, L.coarse, mp, cap);
+      if (form && got == MGLMA_ERR_OOM) {
+        MG_CUDA(cudaStreamSynchronize(s));
+        eng[l]->copies.drop();
+        eng[l].reset();
+        MG_CUDA(cudaStreamSynchronize(s));
+        MG_CUDA(cudaMemPoolTrimTo(ctx->pool, 0));
+      }
+    }
+    if (got == MGLMA_ERR_OOM && cap < 1)
+      return fail(MGLMA_ERR_OOM, "serve: not enough free HBM for one slot of lattice " + std::to_string(l));
+    MG_CHECK(got);
     st.slots[l] = cap;
     st.slot_bytes[l] = (double)per;
   }

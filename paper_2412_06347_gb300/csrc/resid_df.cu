@@ -216,19 +216,26 @@ __global__ void split_df_kernel(const double2* __restrict__ in, float4* __restri
   out[i] = make_float4(a.hi, a.lo, b.hi, b.lo);
 }
 
-static mglma_status gauge_df_ready(mglma_gauge_s* G, cudaStream_t s) {
+mglma_status gauge_df_ready(mglma_gauge_s* G, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(G->eo_mu);
   if (G->Udf && G->Cdf) return MGLMA_OK;
-  const size_t V = (size_t)G->g.V, nu = 36 * V, nc = 36 * V;
-  if (!G->Udf) {
-    MG_CUDA(cudaMalloc(&G->Udf, nu * sizeof(float4)));
-    split_df_kernel<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(G->U64, G->Udf, nu);
-    MG_LAUNCH_CHECK();
+  const size_t n = 36 * (size_t)G->g.V;  // link components, pairs of clover reals
+  cudaError_t e = cudaMalloc(&G->Udf, n * sizeof(float4));
+  if (!e) e = cudaMalloc(&G->Cdf, n * sizeof(float4));
+  if (!e) {
+    split_df_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(G->U64, G->Udf, n);
+    split_df_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(G->C64, G->Cdf, n);
+    e = cudaGetLastError();
+    if (!e) e = cudaStreamSynchronize(s);  // other streams use them without waiting
+    if (!e) return MGLMA_OK;
   }
-  if (!G->Cdf) {
-    MG_CUDA(cudaMalloc(&G->Cdf, nc * sizeof(float4)));
-    split_df_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(G->C64, G->Cdf, nc);
-    MG_LAUNCH_CHECK();
-  }
+  cudaGetLastError();
+  cudaFree(G->Udf);
+  cudaFree(G->Cdf);
+  G->Udf = G->Cdf = nullptr;
+  if (e == cudaErrorMemoryAllocation)
+    return fail(MGLMA_ERR_OOM, "mg solve: no memory for the double-float links and clover");
+  MG_CUDA(e);
   return MGLMA_OK;
 }
 

@@ -812,8 +812,8 @@ __global__ void eo_extract_kernel(const float4* __restrict__ f, float4* __restri
 }
 
 // ============================================================ host side
-mglma_status fine_eo_ready(mglma_ctx ctx, mglma_gauge_s* G, bool* usable, cudaStream_t s) {
-  std::lock_guard<std::mutex> lock(G->eo_mu);
+// fine_eo_ready with eo_mu held
+static mglma_status form_copies(mglma_ctx ctx, mglma_gauge_s* G, bool* usable, cudaStream_t s) {
   *usable = false;
   if (G->eo_state < 0) return MGLMA_OK;
   if (G->eo_state > 0) {
@@ -865,6 +865,36 @@ mglma_status fine_eo_ready(mglma_ctx ctx, mglma_gauge_s* G, bool* usable, cudaSt
   }
   MG_CUDA(e);
   return MGLMA_OK;
+}
+
+mglma_status fine_eo_ready(mglma_ctx ctx, mglma_gauge_s* G, bool* usable, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(G->eo_mu);
+  return form_copies(ctx, G, usable, s);
+}
+
+mglma_status EoUse::acquire(mglma_ctx ctx, const mglma_gauge_s* g, cudaStream_t s) {
+  mglma_gauge_s* gg = const_cast<mglma_gauge_s*>(g);
+  std::lock_guard<std::mutex> lock(gg->eo_mu);
+  MG_CHECK(form_copies(ctx, gg, &usable, s));
+  if (usable) {
+    G = gg;
+    ++G->eo_users;
+  }
+  return MGLMA_OK;
+}
+
+void EoUse::release(bool free) {
+  if (!G) return;
+  std::lock_guard<std::mutex> lock(G->eo_mu);
+  if (--G->eo_users == 0 && free) {
+    cudaFree(G->Ueo);
+    cudaFree(G->Ceo);
+    cudaFree(G->Ieo);
+    G->Ueo = G->Ceo = G->Ieo = nullptr;
+    G->eo_state = 0;
+  }
+  G = nullptr;
+  usable = false;
 }
 
 static EoLinks eo_links(const mglma_gauge_s* G) { return EoLinks{G->Ueo}; }

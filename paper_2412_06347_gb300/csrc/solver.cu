@@ -302,13 +302,18 @@ mglma_status mglma_solve_batch(mglma_ctx ctx, mglma_gauge G, mglma_coarse C, con
   // (a batch must not shrink because the library's cache grew).
   int cap = prm->max_batch > 0 ? prm->max_batch : 64;
   if (prm->max_batch <= 0) {
-    size_t room = device_room(ctx, s);
-    // the multigrid solve's double-float links and clover (2 x 36 float4 per
-    // site), made on its first use, come out of the same room
-    if (prm->method == MGLMA_SOLVER_MG && !(G->Udf && G->Cdf)) room -= std::min(room, (size_t)V * 1152);
-    // and the even-odd stencil's links and clover
-    if (prm->method == MGLMA_SOLVER_MG && G->eo_state == 0) room -= std::min(room, (size_t)V * 576);
-    const size_t per_site = prm->method != MGLMA_SOLVER_MG ? 6 * 192 : 4 * 192 + (size_t)(7 + 2 * prm->gcr_m) * 96;
+    // the multigrid solve's copies of links and clover, made on its first use, come
+    // out of the same room
+    bool even_odd = false;
+    if (prm->method == MGLMA_SOLVER_MG) {
+      MG_CHECK(gauge_df_ready(G, s));
+      MG_CHECK(fine_eo_ready(ctx, G, &even_odd, s));
+    }
+    const size_t room = device_room(ctx, s);
+    const size_t per_site = prm->method != MGLMA_SOLVER_MG
+                                ? 6 * 192
+                                : mg_site_bytes(even_odd, prm->gcr_m, prm->nu,
+                                                dslash_mr_fused(ctx, G, std::min(total, 64)));
     const size_t per_rhs = per_site * (size_t)V;
     cap = (int)std::max<size_t>(1, std::min<size_t>(64, (size_t)(0.7 * (double)room) / per_rhs));
   }

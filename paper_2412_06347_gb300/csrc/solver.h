@@ -80,6 +80,9 @@ struct MgParams {
 // the MG fields of the public parameter block
 MgParams mg_params(const mglma_solve_params& p);
 
+// device bytes per site and RHS of mg_solve's fields (b, x and r with them; its
+// coarse fields are a few per cent of that)
+size_t mg_site_bytes(bool even_odd, int gcr_m, int nu, bool bf16_smoother);
 mglma_status mg_solve(mglma_ctx ctx, const mglma_gauge_s* G, const mglma_coarse_s* C, const Spinor& b, Spinor& x,
                       const MgParams& p, std::vector<RhsStat>& out, cudaStream_t s);
 mglma_status coarse_solve64(mglma_ctx ctx, const mglma_coarse_s* C, const void* b1, void* X, int n, double tol,
