@@ -19,47 +19,11 @@
 namespace mglma {
 namespace {
 
-// packed FP32 pairs; each operation rounds once per lane and is never contracted
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// packed FP32 pairs; the double-float operations on them are df.cuh's
 __device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 pdup(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b, pdup(-1.f), a); }
 __device__ __forceinline__ float2 pswap(float2 a, bool s) { return s ? make_float2(a.y, a.x) : a; }
-
-// two double-floats, lane by lane (df.cuh gives the operations and their errors)
-struct DF2 {
-  float2 hi, lo;
-};
-__device__ __forceinline__ DF2 two_sum2(float2 a, float2 b) {
-  const float2 s = padd(a, b), bb = psub(s, a);
-  return DF2{s, padd(psub(a, psub(s, bb)), psub(b, bb))};
-}
-__device__ __forceinline__ DF2 fast_two_sum2(float2 a, float2 b) {
-  const float2 s = padd(a, b);
-  return DF2{s, psub(b, psub(s, a))};
-}
-__device__ __forceinline__ DF2 add2(DF2 x, DF2 y) {
-  const DF2 s = two_sum2(x.hi, y.hi);
-  return fast_two_sum2(s.hi, padd(s.lo, padd(x.lo, y.lo)));
-}
-// x y + z for x = (xh, xl) per lane
-__device__ __forceinline__ DF2 fma2(float2 xh, float2 xl, DF2 y, DF2 z) {
-  const float2 nh = make_float2(-xh.x, -xh.y), nl = make_float2(-xl.x, -xl.y);
-  const float2 p = pmul(xh, y.hi);
-  // minus the product's rounding error and its cross terms
-  const float2 t = pfma(nh, y.lo, pfma(nl, y.hi, pfma(nh, y.hi, p)));
-  const DF2 s = two_sum2(p, z.hi);
-  return fast_two_sum2(s.hi, padd(s.lo, psub(z.lo, t)));
-}
-// the same for FP32 y
-__device__ __forceinline__ DF2 fma2(float2 xh, float2 xl, float2 y, DF2 z) {
-  const float2 nh = make_float2(-xh.x, -xh.y), nl = make_float2(-xl.x, -xl.y);
-  const float2 p = pmul(xh, y);
-  const float2 t = pfma(nl, y, pfma(nh, y, p));
-  const DF2 s = two_sum2(p, z.hi);
-  return fast_two_sum2(s.hi, padd(s.lo, psub(z.lo, t)));
-}
+__device__ __forceinline__ float2 pneg(float2 a) { return make_float2(-a.x, -a.y); }
 
 struct CD2 {
   DF2 re, im;
@@ -78,7 +42,7 @@ __global__ void __launch_bounds__(128, 3) resid_df_kernel(const float4* __restri
   int x[4];
   site_coords(q, site, x);
   const float4* er = e + (size_t)rhs * 6 * V;
-  const DF2 zero{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const DF2 zero;
   CD2 up[3], lw[3];  // sums of the hops over spins (0, 1) and (2, 3), per colour
 #pragma unroll
   for (int c = 0; c < 3; ++c) up[c] = lw[c] = CD2{zero, zero};
@@ -108,8 +72,8 @@ __global__ void __launch_bounds__(128, 3) resid_df_kernel(const float4* __restri
         const float2 u0 = comp(c), u1 = comp(3 + c), l0 = comp(6 + c), l1 = comp(9 + c);
         const float2 lr = pswap(make_float2(l0.x, l1.x), sw), li = pswap(make_float2(l0.y, l1.y), sw);
         const float2 tr = im ? make_float2(-li.x, -li.y) : lr, ti = im ? lr : li;
-        hp[c].re = two_sum2(pmul(pdup(bs), make_float2(u0.x, u1.x)), pmul(pmul(pdup(bs), f), tr));
-        hp[c].im = two_sum2(pmul(pdup(bs), make_float2(u0.y, u1.y)), pmul(pmul(pdup(bs), f), ti));
+        hp[c].re = dfl::two_sum(pmul(pdup(bs), make_float2(u0.x, u1.x)), pmul(pmul(pdup(bs), f), tr));
+        hp[c].im = dfl::two_sum(pmul(pdup(bs), make_float2(u0.y, u1.y)), pmul(pmul(pdup(bs), f), ti));
       }
     }
     const float4* ul = U + (size_t)mu * 9 * V + (fwd ? site : n);
@@ -125,20 +89,20 @@ __global__ void __launch_bounds__(128, 3) resid_df_kernel(const float4* __restri
         const float4 w = __ldg(ul + (size_t)(a * ra + b * rb) * V);  // re.hi, re.lo, im.hi, im.lo
         const float2 rh = pdup(w.x), rl = pdup(w.y), ih = pdup(sg * w.z), il = pdup(sg * w.w);
         const float2 mh = pdup(-sg * w.z), ml = pdup(-sg * w.w);
-        g.re = fma2(rh, rl, hp[b].re, g.re);
-        g.re = fma2(mh, ml, hp[b].im, g.re);
-        g.im = fma2(rh, rl, hp[b].im, g.im);
-        g.im = fma2(ih, il, hp[b].re, g.im);
+        g.re = fma(DF2(rh, rl), hp[b].re, g.re);
+        g.re = fma(DF2(mh, ml), hp[b].im, g.re);
+        g.im = fma(DF2(rh, rl), hp[b].im, g.im);
+        g.im = fma(DF2(ih, il), hp[b].re, g.im);
       }
-      up[a].re = add2(up[a].re, g.re);
-      up[a].im = add2(up[a].im, g.im);
+      up[a].re = up[a].re + g.re;
+      up[a].im = up[a].im + g.im;
       auto part = [&](const DF2& v, float f) {
         const float2 m = pmul(pdup(f), sl);
         return DF2{pmul(m, pswap(v.hi, sw)), pmul(m, pswap(v.lo, sw))};
       };
       const DF2 tr = im ? part(g.im, -1.f) : part(g.re, 1.f), ti = im ? part(g.re, 1.f) : part(g.im, 1.f);
-      lw[a].re = add2(lw[a].re, tr);
-      lw[a].im = add2(lw[a].im, ti);
+      lw[a].re = lw[a].re + tr;
+      lw[a].im = lw[a].im + ti;
     }
   }
   // D e = A e - hops / 2; lanes now pair component k with 6 + k
@@ -171,8 +135,8 @@ __global__ void __launch_bounds__(128, 3) resid_df_kernel(const float4* __restri
     CD2 o{pick(up[c].re, lw[c].re), pick(up[c].im, lw[c].im)};
     float2 dh, dl;
     elem(i, dh, dl);
-    o.re = fma2(dh, dl, pr[i], o.re);
-    o.im = fma2(dh, dl, pi[i], o.im);
+    o.re = fma(DF2(dh, dl), pr[i], o.re);
+    o.im = fma(DF2(dh, dl), pi[i], o.im);
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
       if (j == i) continue;
@@ -181,13 +145,13 @@ __global__ void __launch_bounds__(128, 3) resid_df_kernel(const float4* __restri
       elem(k, rh, rl);
       elem(k + 1, ih, il);
       if (i > j) {  // conjugate element
-        ih = make_float2(-ih.x, -ih.y);
-        il = make_float2(-il.x, -il.y);
+        ih = pneg(ih);
+        il = pneg(il);
       }
-      o.re = fma2(rh, rl, pr[j], o.re);
-      o.re = fma2(make_float2(-ih.x, -ih.y), make_float2(-il.x, -il.y), pi[j], o.re);
-      o.im = fma2(rh, rl, pi[j], o.im);
-      o.im = fma2(ih, il, pr[j], o.im);
+      o.re = fma(DF2(rh, rl), pr[j], o.re);
+      o.re = fma(DF2(pneg(ih), pneg(il)), pi[j], o.re);
+      o.im = fma(DF2(rh, rl), pi[j], o.im);
+      o.im = fma(DF2(ih, il), pr[j], o.im);
     }
     bool other = false;
     auto sum = [&](float hi, float lo) { return f2d_fast(hi, other) + f2d_fast(lo, other); };
