@@ -926,7 +926,7 @@ struct TwoLevel {
     const int64_t V = C->sub->geo.V;
     MG_CHECK(dalloc(ctx, (void**)&part,
                     (eo ? schur_part_doubles(V, n) : dslash_dot_part_doubles(V, n)) * sizeof(double), s));
-    MG_CHECK(sc.alloc(ctx, n, 1, eo ? kGroup + 1 : 1, s));
+    MG_CHECK(sc.alloc(ctx, n, 1, eo ? kGroup : 1, s));
     cs.ctx = ctx;
     cs.s = s;
     cs.C = C;
@@ -1054,14 +1054,10 @@ struct TwoLevel {
       Spinor sk = slot(k - 1), sn = slot(k);
       MG_CHECK(schur_odd(ctx, G, *tc, w, s));
       if (k % kGroup == 0) {
-        // the next slot reuses the group's first: its sum goes into z first,
-        // its last alpha moves out of the way of the new group
+        // the next slot reuses the group's first: its sum goes into z first
         MG_CHECK(mr_iterate(ctx, z, sv.p, sv.prec, stride, kGroup, al, s));
-        MG_CUDA(cudaMemcpyAsync(al + (size_t)kGroup * n, alpha(k - 1), sizeof(float2) * n, cudaMemcpyDeviceToDevice, s));
-        MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, al + (size_t)kGroup * n, alpha(k), part, s));
-      } else {
-        MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, alpha(k - 1), alpha(k), part, s));
       }
+      MG_CHECK(schur_mr_step(ctx, G, w, *tc, *tn, sk, sn, alpha(k - 1), alpha(k), part, s));
       std::swap(tc, tn);
     }
     return mr_iterate(ctx, z, sv.p, sv.prec, stride, (steps - 1) % kGroup + 1, al, s);
