@@ -1,16 +1,17 @@
-// Inverse of a packed Hermitian 6x6 clover block in registers (one thread).
+// Inverse of a packed Hermitian 6x6 clover block (one thread).
 #pragma once
 #include "stencil.cuh"
 
 namespace mglma {
 
-// ci = c^-1 by Gauss-Jordan with partial pivoting in FP64; the inverse of a
+// pk = c^-1 by Gauss-Jordan with partial pivoting in FP64; the inverse of a
 // Hermitian matrix is Hermitian and is packed the same way.  Every loop is
 // unrolled and every index static (row and column exchanges are predicated
-// swaps), so the 6x6 matrix stays in registers: a version that indexed a
-// local array by the pivot row gave wrong inverses when built with -O3 on
-// sm_103a (exact in a debug build and on the host).  False when the block is
-// singular.
+// swaps); ptxas keeps 576 bytes of it in local memory all the same (254 registers),
+// which a set-up kernel can afford.  An earlier version that indexed the array by
+// the pivot row gave wrong inverses under -O3 for a cause never found;
+// tests/test_gpu_clover_inverse.py holds blocks whose rows are exchanged.  False
+// when the block is singular.
 __device__ __forceinline__ bool clover_inverse6(const double c[36], double pk[36]) {
   Cx<double> M[6][6];
 #pragma unroll
