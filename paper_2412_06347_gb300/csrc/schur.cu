@@ -442,18 +442,35 @@ struct EvArgs {
 };
 
 // per-thread sums of one site each added over the CTA's warp in FP32 (the FP64 pipe
-// of GB300 is too narrow for a per-thread FP64 tree) and to acc in FP64: FP32
-// never carries more than the 32 sites of a warp, whatever nsub is
+// of GB300 is too narrow for a per-thread FP64 tree); FP32 never carries more than
+// the 32 sites of a warp, whatever nsub is.  The values are halved between the
+// lanes while there are several (six values: 9 shuffles instead of 30), so a lane
+// ends with the total of value warp_value(lane)
 template <int NV>
-__device__ __forceinline__ void warp_partials(float* v, double* acc) {
-  static_assert(SCHUR_T == 32, "one warp per CTA");
+__device__ __forceinline__ float warp_total(const float (&v)[NV]) {
+  static_assert(SCHUR_T == 32 && NV <= 8, "one warp per CTA");
+  constexpr int P = NV <= 4 ? 4 : 8;
+  float a[P];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
+  for (int i = 0; i < P; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.f;
+  int o = 16;
 #pragma unroll
-    for (int e = 0; e < NV; ++e) v[e] += __shfl_down_sync(0xffffffffu, v[e], o);
-  if (threadIdx.x == 0)
+  for (int n = P; n > 1; n /= 2, o /= 2) {
+    const bool up = threadIdx.x & o;
 #pragma unroll
-    for (int e = 0; e < NV; ++e) acc[e] += (double)v[e];
+    for (int i = 0; i < n / 2; ++i) {
+      const float keep = up ? a[i + n / 2] : a[i], send = up ? a[i] : a[i + n / 2];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (int q = 16 / P; q > 0; q /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], q);
+  return a[0];
+}
+// the value whose total a lane holds; the first lane of each group of 32 / P writes
+template <int NV>
+__device__ __forceinline__ int warp_value(int lane) {
+  return lane / (NV <= 4 ? 8 : 4);
 }
 
 // SM: storage of the smoother's fields, SpinBf16 or float
@@ -467,17 +484,14 @@ __global__ void __launch_bounds__(SCHUR_T, schur_ctas<EV>())
   using SX = typename std::conditional<EV == EV_DOT || EV == EV_MR, SM, float>::type;
   const EoTile t(g, nrhs);
   const int r = t.r;
-  __shared__ double sum[NV];  // thread 0's
-  if (RED && threadIdx.x == 0)
-#pragma unroll
-    for (int e = 0; e < NV; ++e) sum[e] = 0.0;
+  double sum = 0.0;  // of value warp_value(lane)
   for (int k = 0; k < nsub; ++k) {
     const uint32_t u0 = (t.blk * nsub + k) * SCHUR_T, u = u0 + threadIdx.x;
-    if (u0 >= g.Vh) break;
+    if (RED ? u0 >= g.Vh : u >= g.Vh) break;
     float v[NV];
 #pragma unroll
     for (int e = 0; e < NV; ++e) v[e] = 0.f;
-    if (u < g.Vh) {
+    if (!RED || u < g.Vh) {
       float2 acc[12];
       hops2<float>(g, u, 0, U, rhs_of<float>(w, g, r), acc);
       if (EV == EV_PREP) {
@@ -596,12 +610,13 @@ __global__ void __launch_bounds__(SCHUR_T, schur_ctas<EV>())
     }
     if (RED) {
       __syncwarp();
-      warp_partials<NV>(v, sum);
+      sum += (double)warp_total(v);
     }
   }
   if (RED) {
-    __syncwarp();
-    if (threadIdx.x < NV) a.part[((size_t)r * eo_blocks(g.Vh) + t.blk) * NV + threadIdx.x] = sum[threadIdx.x];
+    const int e = warp_value<NV>(threadIdx.x);
+    if (threadIdx.x % (NV <= 4 ? 8 : 4) == 0 && e < NV)
+      a.part[((size_t)r * eo_blocks(g.Vh) + t.blk) * NV + e] = sum;
   }
 }
 
