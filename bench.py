@@ -61,12 +61,11 @@ C5 = dict(shapes=[(128, 64, 64, 64), (96, 48, 48, 48), (64, 32, 32, 32)], eps=0.
 
 
 # DRAM traffic per lattice site of one launch of a kernel class at a given
-# RHS count, from ncu (dram__bytes_read.sum + dram__bytes_write.sum of one
-# capture divided by the captured lattice's volume; traffic grows with the
-# volume).  Reported only while the class's kernels are the ones captured: the
-# even-odd passes that the solve launches have no capture at this size, so the
-# table is empty and `traffic` null.
-NCU_TRAFFIC_PER_SITE = {}
+# RHS count, from ncu (dram__bytes_read.sum + dram__bytes_write.sum divided by
+# the captured lattice's volume; traffic grows with the volume).  The even-odd
+# passes on 16x32^3, averaged over the twelve launches of an FGCR iteration
+# (profiles/schur_32x16x16x16_nrhs16.md).
+NCU_TRAFFIC_PER_SITE = {("dslash32", 16): 2683.0}
 
 
 def peaks():

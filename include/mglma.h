@@ -317,7 +317,10 @@ mglma_status mglma_coarse_prolong(mglma_ctx ctx, mglma_coarse level, int nrhs, c
  * calT_l Q_l^-1 calR_l gamma5 = calT_l D_l^-1 calR_l).  levels[0] is a
  * level-1 operator of g's basis and levels[k] the mglma_coarse_build_next
  * child of levels[k-1]; each D_l^-1 is solved to relative residual tol by
- * FP64 defect correction around FP32 GCR on that level's stored operator.
+ * flexible GCR on the level's FP64 operator, preconditioned by loose FP32 solves
+ * on the stored one; what that leaves above tol, by FP64 defect correction
+ * around FP32 GCR.  Every RHS follows its own recurrence, as in
+ * mglma_solve_batch.
  * With x = D^-1 b from mglma_solve_batch: S_0 b = x - psi[0], S_l b =
  * psi[l-1] - psi[l], S_{N-1} b = psi[N-2] (N = nlevels + 1 levels in all).
  *   b: nrhs canonical spinors; psi: nlevels x nrhs canonical spinors
@@ -485,7 +488,7 @@ void mglma_solve_params_default(mglma_solve_params* p, int method);
  * not depend on the batch it is in.  coarse may be NULL for MGLMA_SOLVER_CGNE.
  * x_coarse (nullable): also returns the coarse-space piece
  *   psi1 = T0 D1^-1 R0 b (S1 b of Sec. 2 via App. chirality), with D1^-1
- *   solved to tol by FP64 defect correction; S0 b = x - psi1.
+ *   solved to tol / 10 as in mglma_pieces; S0 b = x - psi1.
  * stats (nullable): one entry per RHS.
  * Returns MGLMA_ERR_NOT_CONVERGED (best iterate in x) if any RHS misses tol. */
 mglma_status mglma_solve_batch(mglma_ctx ctx, mglma_gauge g, mglma_coarse coarse, const mglma_solve_params* params,

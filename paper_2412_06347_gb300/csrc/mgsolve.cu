@@ -10,11 +10,15 @@
 //     z += MR(D, r - D z)    (minimal-residual smoothing steps)
 // With every extent even the inner system is the even-odd one, S x_e = b' on
 // half-lattice fields (schur.cu), smoothed by (nu + 1) / 2 steps on S: a step on
-// S costs what one on D does and damps about what two do.  Steps on S against
-// the solve's time, 64x32^3, 16 RHS, to 1e-12, after the first version: 2 / 3 /
-// 4 / 5 / 7 -> 1192 / 1076 / 1158 / 1126 / 1271 ms (16 RHS of 32x16^3: 112 / 91 /
-// 81 / 81 / 80; one of 8^4: 26.6 / 20.1 / 17.7 / 15.5 / 12.6).  An odd extent
-// keeps the full system and nu steps on D.
+// S costs what one on D does and damps about what two do, so a caller's nu keeps
+// its meaning.  That is the rule's reason; it is not the fastest count at every
+// size.  ms to 1e-12 with 2 / 3 / 4 (the default nu) / 5 / 6 / 7 / 8 steps on S:
+//   1 RHS of 8^4       22.3 / 17.0 / 15.0 / 13.3 / 11.3 / 10.5 / 9.8
+//   4 of 16^4          44.6 / 35.7 / 32.2 / 31.5 / 30.9 / 28.2 / 28.9
+//   12 of 32x16^3      91.8 / 74.9 / 67.3 / 67.8 / 72.7 / 67.0 / 65.6
+//   8 of 48x24^3       228 / 205 / 196 / 201 / 195 / 196 / 180
+//   16 of 64x32^3      966 / 874 / 948 / 925 / 990 / 1055 / 1120
+// An odd extent keeps the full system and nu steps on D.
 // The pieces of Sec. 2: psi1 = T0 D1^-1 R0 b with D1^-1 solved to tol by an
 // FP64 flexible GCR on the coarse operator (defect correction as a fallback),
 // psi0 = x - psi1 (App. chirality: T Q1^-1 R gamma5 = T D1^-1 R when [P, gamma5]

@@ -17,9 +17,10 @@
 //              dots, a whole MR step) in the epilogue.
 // w is FP32; x is FP32, or BF16 for the smoother's fields (FP32 too when asked for).
 //
-// What bounds it: nothing alone.  ncu on 32^4, 16 RHS (odd pass, BF16 in): FMA
-// pipe 50 %, issue slots 49 %, L1 51 %, DRAM 37 %, long-scoreboard stalls 4.5
-// of 7.7 warp cycles per instruction; 10 to 16 warps per SM measure the same.
+// What bounds it: nothing alone.  ncu on 32x16^3, 16 RHS, odd pass with BF16 in /
+// even pass of an MR step: issue slots 46 / 39 %, L1 49 / 46 %, DRAM 27 / 37 %, and
+// 4.2 / 5.7 warp cycles per instruction wait on loads; 10 to 16 warps per SM measure
+// the same.
 // The full-lattice stencil it replaces issued 2717 instructions per site and
 // RHS; the odd pass issues 1412.  Complex products run as packed FP32 pairs (one
 // FFMA2 does (re, im) with a duplicated link real, so a 3x3 complex product is 18
@@ -28,9 +29,10 @@
 // with the time-boundary sign applied (no third row to rebuild, no hop factor:
 // -1/2 rides on the stored inverse clover and on one packed FMA per component),
 // and links and clover are parity-split so a warp reads whole sectors.
-// 64x32^3, 16 RHS, us: odd pass BF16 1207 / FP32 1373, even pass MR step 1722,
-// dot 1470, FGCR image 1630; one MR step on S (2929) against 3500 for one on D
-// that damps about half as much.  A whole solve to 1e-12: 1507 -> 1102 ms.
+// 64x32^3, 16 RHS, us: odd pass BF16 1185 / FP32 1345, even pass MR step 1683,
+// dot 1546, FGCR image 1790 (one earlier image; 2301 with three); one MR step on S
+// (2868) against 3500 for one on D that damps about half as much.  A whole solve to
+// 1e-12, when this form came in: 1507 -> 1102 ms.
 //
 // Fields of one parity: [rhs][6][Vh] float4 (FP32) or [rhs][3][Vh] uint4
 // (BF16), Vh = V / 2, site x at index x >> 1.  A row's address is uniform in
